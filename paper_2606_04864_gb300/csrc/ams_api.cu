@@ -145,12 +145,13 @@ struct ams_handle_s {
     int64_t fac_elems = 0;
     // reduced-precision local factors in the TMA tile layout
     bool use_tma = false;
-    float *d_tfwd = nullptr, *d_tbwd = nullptr, *d_piv = nullptr;
-    int64_t* d_trow0 = nullptr;
-    int64_t tile_elems = 0;
-    CUtensorMap tmF{}, tmB{};
+    float *d_tfwd = nullptr, *d_tmma = nullptr, *d_piv = nullptr;
+    int64_t *d_trow0 = nullptr, *d_toff = nullptr, *d_brow0 = nullptr;
+    int64_t tile_elems = 0, nbrows = 0;
+    CUtensorMap tmF{};
     double* d_psi64 = nullptr;
     void* d_psi = nullptr;              // basis in the solve precision
+    void* d_psif = nullptr;             // the same in MMA fragment order (reduced precision)
     int64_t psi_elems = 0;
     CoarseItem *d_fwd = nullptr, *d_bwd = nullptr;
     int nfwd = 0, nbwd = 0;
@@ -457,30 +458,31 @@ static ams_status build_local_factors(ams_handle h, const int64_t* d_rowptr, con
     launch_band_cholesky(ba, d_band, d_status);
     void* fac = nullptr;
     if (tiles) {
-        // forward/backward FP32 tiles (c tiles per block row) + pivots
-        std::vector<int64_t> toff(h->N), trow0(h->N);
+        // FP32 tiles (c per block row) in the two kernels' orders + pivots
+        std::vector<int64_t> toff(h->N), trow0(h->N), brow0(h->N);
         int64_t ttot = 0;
+        h->nbrows = 0;
         for (int s = 0; s < h->N; ++s) {
             toff[s] = ttot;
             trow0[s] = ttot / 32;
+            brow0[s] = h->nbrows;
             ttot += (int64_t)h->h_subs[s].nb * h->h_subs[s].c * 1024;
+            h->nbrows += h->h_subs[s].nb;
         }
-        int64_t* d_toff = nullptr;
-        AMS_TRY(upload(h, &d_toff, toff));
+        AMS_TRY(upload(h, &h->d_toff, toff));
         AMS_TRY(upload(h, &h->d_trow0, trow0));
+        AMS_TRY(upload(h, &h->d_brow0, brow0));
         AMS_TRY(h->alloc_t(&h->d_tfwd, (size_t)ttot));
-        AMS_TRY(h->alloc_t(&h->d_tbwd, (size_t)ttot));
+        AMS_TRY(h->alloc_t(&h->d_tmma, (size_t)ttot));
         AMS_TRY(h->alloc_t(&h->d_piv, (size_t)h->n_pad));
-        launch_band_pack_tiles(h->stream, (int)work.size(), h->d_subs, d_band_off, d_work, d_band, d_toff,
-                               h->d_tfwd, h->d_tbwd, h->d_piv);
+        launch_band_pack_tiles(h->stream, (int)work.size(), h->d_subs, d_band_off, d_work, d_band, h->d_toff,
+                               h->d_tfwd, h->d_tmma, h->d_piv);
         AMS_CUDA_TRY(cudaGetLastError());
         AMS_CUDA_TRY(make_tile_map(h->d_tfwd, ttot / 32, &h->tmF));
-        AMS_CUDA_TRY(make_tile_map(h->d_tbwd, ttot / 32, &h->tmB));
         h->tile_elems = ttot;
         h->use_tma = true;
         fac_tot = 0;
         AMS_CUDA_TRY(cudaStreamSynchronize(h->stream));
-        h->release(d_toff);
     } else {
         AMS_TRY(h->alloc(&fac, (size_t)fac_tot * (out_fp64 ? 8 : 4)));
         launch_band_pack_work(h->stream, (int)work.size(), h->d_subs, d_band_off, d_work, d_band, d_fac_off,
@@ -1163,6 +1165,10 @@ static ams_status setup_impl(int32_t nsys, const ams_system_desc* systems, const
         if (h->prec == AMS_PREC_FP64)
             AMS_CUDA_TRY(cudaMemcpyAsync(h->d_psi, h->d_psi64, sizeof(double) * h->psi_elems,
                                          cudaMemcpyDeviceToDevice, h->stream));
+        if (h->use_tma && h->mmax > 0) {
+            AMS_TRY(h->alloc(&h->d_psif, (size_t)h->nbrows * local_mma_psi_words(h->prec, h->mmax) * 16));
+            launch_pack_psi(h->stream, h->N, h->d_subs, h->d_brow0, h->prec, h->mmax, h->d_psi, h->d_psif);
+        }
         AMS_CUDA_TRY(cudaGetLastError());
         if (h->mmax > 0) AMS_TRY(setup_coarse(H, inputs, d_irp, d_icol, d_ival, d_psi_used));
         h->release(d_psi_used);
@@ -1296,7 +1302,7 @@ static int64_t spin_budget(ams_handle h) {
 
 // Fine-level local solves (+ restriction when the coarse space exists).
 static LocalTmaArgs local_tma_args(ams_handle h, int ld, const ResidIn& in, bool with_state) {
-    LocalTmaArgs a{h->stream, h->N, h->d_subs, &h->tmF, &h->tmB, h->d_trow0, h->d_piv, in, ld, h->cmax,
+    LocalTmaArgs a{h->stream, h->N, h->d_subs, &h->tmF, h->d_trow0, h->d_tmma, h->d_toff, h->d_brow0, h->d_piv, in, ld, h->cmax,
                    std::max(1, h->mmax), h->nbmax, spin_budget(h), with_state ? h->d_st : nullptr,
                    h->use_pdl, h->tune[ld].depth, h->tune[ld].nr, h->tune[ld].l2mode, h->tune[ld].l2keep,
                    &h->d_st->status, h->opt.timeout_probe};
@@ -1311,7 +1317,7 @@ static LocalTmaArgs local_tma_args(ams_handle h, int ld, const ResidIn& in, bool
 // Launches of one local-solve pass beyond the first: the several-RHS
 // kernel launches once per band-width group.
 static int local_extra_launches(ams_handle h, int ld) {
-    return (h->use_tma && ld >= 8 && h->cls_c.size() > 1) ? (int)h->cls_c.size() - 1 : 0;
+    return (h->use_tma && ld >= 2 && h->cls_c.size() > 1) ? (int)h->cls_c.size() - 1 : 0;
 }
 
 static ams_status launch_local(ams_handle h, int ld, const ResidIn& in, bool with_state,
@@ -1319,7 +1325,7 @@ static ams_status launch_local(ams_handle h, int ld, const ResidIn& in, bool wit
     const bool coarse = h->Nc > 0 && restrict_rc;
     if (h->use_tma) {
         LocalTmaArgs a = local_tma_args(h, ld, in, with_state);
-        AMS_CUDA_TRY(launch_local_tma(a, h->prec, h->d_psi, h->d_zf, coarse ? h->d_rc : nullptr));
+        AMS_CUDA_TRY(launch_local_tma(a, h->prec, h->d_psi, h->d_psif, h->d_zf, coarse ? h->d_rc : nullptr));
     } else {
         LocalSolveArgs la{h->stream, h->N, h->d_subs, in, nullptr, ld, h->cmax, std::max(1, h->mmax),
                           with_state ? h->d_st : nullptr, h->use_pdl, h->tune[ld].depth};
@@ -1769,15 +1775,11 @@ static ams_status autotune(ams_handle h, const double* f_dev, int nrhs, int ld) 
         T.l2mode = cand[arg][0];
         T.l2keep = cand[arg][1];
     }
-    if (h->use_tma && ld > 1) {   // several-RHS local solve: right-hand sides per warp
+    if (h->use_tma && ld >= 16) {   // several-RHS local solve: right-hand sides per column group
         const ResidIn in{h->d_r, h->d_q, h->d_sc};
         float best = 1e30f;
         int arg = 0;
-        // tensor-core kernel from 8 right-hand sides on: 8 or 16 per warp,
-        // at most four warps; below that 2, 4 or 8 per warp, at most eight
-        const int hi = ld >= 8 ? 16 : 8, lo = ld >= 8 ? 8 : 2, maxw = ld >= 8 ? 4 : 8;
-        for (int nr = hi; nr >= lo; nr /= 2) {
-            if (nr > ld || ld / nr > maxw) continue;
+        for (int nr = 16; nr >= 8; nr /= 2) {
             T.nr = nr;
             float ms = 0.f;
             AMS_TRY(timed_after(spmv, [&]() -> ams_status { return launch_local(h, ld, in, true); }, &ms));

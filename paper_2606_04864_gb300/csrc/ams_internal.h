@@ -57,6 +57,15 @@ struct SubInfo {
 __host__ __device__ inline int64_t blockrow_elems(int c) { return (int64_t)c * 1024 + 32; }
 __host__ __device__ inline int tile_idx(int r, int q) { return q * 32 + (r ^ q); }
 
+// Element (r, q) of a 32x32 FP32 tile in the order of the MMA local solve
+// (k_local_mma.cu): 2x2 micro-tiles (T00, T10, T01, T11) of 16 bytes,
+// micro-row R at 64 R floats, its micro-columns permuted so that fragment
+// loads of the tile and of its transpose touch every bank once.
+__host__ __device__ inline int mma_tile_off(int r, int q) {
+    const int R = r >> 1, Q = q >> 1;
+    return R * 64 + ((Q ^ (((R & 1) << 2) | (R & 2))) << 2) + (r & 1) + 2 * (q & 1);
+}
+
 // ---- coarse inverse GEMM items ---------------------------------------------
 // out[out0 + r][:] = sum_k Mat[moff + (row_in_node + r)*ldm + k] * in[g(k)][:]
 // over k in [k0, k1), where g maps a node-matrix column to an input row

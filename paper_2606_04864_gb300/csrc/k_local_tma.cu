@@ -2,25 +2,22 @@
 // fine-level term sum_i R_i^T A_i^{-1} R_i r) with the factor tiles fed by
 // the Tensor Memory Accelerator.
 //
-// Storage (FP32, one 32x32 tile = 4 KB, row-major inside a tile):
-//   forward copy,  block row K: [ M_K | L_{K,K-c+1} | ... | L_{K,K-1} ]
-//   backward copy, block row K: [ M_K^T | L_{K,K-c+1}^T | ... ]
-// with M_K[r][q] = L_{K,K-c}[r][q] (q >= r) and (L_KK^{-1})[r][q] (q < r),
-// plus the reciprocal pivots 1/L_KK[r][r] in a per-row array.  Both copies
-// are viewed as 2-D tensors of 32-float rows; one TMA box is one tile,
-// written to shared memory with the 128-byte swizzle (16-byte chunk j of
-// tile row r lands at chunk j ^ (r mod 8)), so a lane that owns tile row r
-// reads its 32 coefficients with eight conflict-free 128-bit loads.  Each
-// ring slot has an mbarrier that the TMA completes (expect-tx); every wait
-// is bounded and a timeout sets AMS_ERR_DEVICE_TIMEOUT.
+// Storage (FP32, one 32x32 tile = 4 KB, row-major inside a tile), block row
+// K: [ M_K | L_{K,K-c+1} | ... | L_{K,K-1} ] with M_K[r][q] = L_{K,K-c}[r][q]
+// (q >= r) and (L_KK^{-1})[r][q] (q < r), plus the reciprocal pivots
+// 1/L_KK[r][r] in a per-row array.  The tiles are viewed as a 2-D tensor of
+// 32-float rows; one TMA box is one tile, written to shared memory with the
+// 128-byte swizzle (16-byte chunk j of tile row r lands at chunk
+// j ^ (r mod 8)), so a lane that owns tile row r reads its 32 coefficients
+// with eight conflict-free 128-bit loads.  Each ring slot has an mbarrier
+// that the TMA completes (expect-tx); every wait is bounded and a timeout
+// sets AMS_ERR_DEVICE_TIMEOUT.
 //
 // Forward sweep (lane = row r of block row K):
 //   t = r_K - sum_d L_{K,K-c+d} y_{K-c+d} ;  y_K = L_KK^{-1} t
-// Backward sweep (lane = column l of block column K, i.e. row l of the
-// transposed tiles):
+// Backward sweep (lane = column l of block column K):
 //   w = y_K - sum_d L_{K+d,K}^T x_{K+d}   ;  x_K = L_KK^{-T} w
 #include <cstdint>
-#include <cstdio>
 
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -31,353 +28,6 @@
 #include "tma.cuh"
 
 namespace ams {
-
-// Row stride (floats) of the y/x ring of the several-RHS kernel: ld + 4 for
-// ld >= 2 (conflict-free per-lane row stores, 16-byte aligned rows); one
-// right-hand side keeps a contiguous vector.
-__host__ __device__ __forceinline__ int local_tma_row_stride(int ld) { return ld >= 2 ? ld + 4 : 1; }
-
-// NR consecutive floats of one ring row (16-byte stores when NR % 4 == 0:
-// eight lanes of a quarter warp then cover all 32 banks).
-template <int NR>
-__device__ __forceinline__ void store_row(float* p, const float (&v)[NR]) {
-    if (NR % 4 == 0) {
-#pragma unroll
-        for (int k = 0; k < NR; k += 4)
-            *reinterpret_cast<float4*>(p + k) = make_float4(v[k], v[(k + 1) % NR], v[(k + 2) % NR], v[(k + 3) % NR]);
-    } else if (NR == 2) {
-        *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1 % NR]);
-    } else {
-#pragma unroll
-        for (int j = 0; j < NR; ++j) p[j] = v[j];
-    }
-}
-
-// Row r of a swizzled 32x32 FP32 tile: 16-byte chunk j (columns 4j..4j+3).
-__device__ __forceinline__ float4 tile_chunk(const float* tile, int r, int j) {
-    return *reinterpret_cast<const float4*>(tile + r * 32 + ((j ^ (r & 7)) << 2));
-}
-__device__ __forceinline__ float f4(const float4& v, int e) {
-    return e == 0 ? v.x : (e == 1 ? v.y : (e == 2 ? v.z : v.w));
-}
-
-// Keep columns q of chunk j with (q >= lo) when upper, (q < lo) otherwise.
-__device__ __forceinline__ float4 mask_chunk(float4 v, int j, int lo, bool upper) {
-    const int q0 = 4 * j;
-    if (upper) {
-        if (q0 + 0 < lo) v.x = 0.f;
-        if (q0 + 1 < lo) v.y = 0.f;
-        if (q0 + 2 < lo) v.z = 0.f;
-        if (q0 + 3 < lo) v.w = 0.f;
-    } else {
-        if (q0 + 0 >= lo) v.x = 0.f;
-        if (q0 + 1 >= lo) v.y = 0.f;
-        if (q0 + 2 >= lo) v.z = 0.f;
-        if (q0 + 3 >= lo) v.w = 0.f;
-    }
-    return v;
-}
-
-// acc[j] += SIGN * sum_q T[row][q] * vec[q*ld + rhs0 + j] over the kept
-// columns.  MODE 0: all; 1: q >= row; 2: q < row; 3: q <= row; 4: q > row.
-template <int NR, int MODE>
-__device__ __forceinline__ void tile_rowdot(const float* tile, int row, const float* vec, int ld, int rhs0,
-                                            float sign, float (&acc)[NR]) {
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        float4 v = tile_chunk(tile, row, j);
-        if (MODE == 1) v = mask_chunk(v, j, row, true);
-        if (MODE == 2) v = mask_chunk(v, j, row, false);
-        if (MODE == 3) v = mask_chunk(v, j, row + 1, false);
-        if (MODE == 4) v = mask_chunk(v, j, row + 1, true);
-        if (NR == 1) {
-            const float4 x = *reinterpret_cast<const float4*>(vec + 4 * j);   // ld == 1
-            acc[0] += sign * (v.x * x.x + v.y * x.y + v.z * x.z + v.w * x.w);
-        } else {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const float cf = sign * f4(v, e);
-                const float* xr = vec + (4 * j + e) * ld + rhs0;
-                if (NR == 2) {
-                    const float2 x = *reinterpret_cast<const float2*>(xr);
-                    acc[0] += cf * x.x;
-                    acc[1 % NR] += cf * x.y;
-                } else {
-#pragma unroll
-                    for (int k = 0; k < NR; k += 4) {
-                        const float4 x = *reinterpret_cast<const float4*>(xr + k);
-                        acc[k + 0] += cf * x.x;
-                        acc[(k + 1) % NR] += cf * x.y;
-                        acc[(k + 2) % NR] += cf * x.z;
-                        acc[(k + 3) % NR] += cf * x.w;
-                    }
-                }
-            }
-        }
-    }
-}
-
-template <typename TP, int NR, int MM>
-__global__ void __launch_bounds__(256)
-k_local_tma(const __grid_constant__ CUtensorMap tmF, const __grid_constant__ CUtensorMap tmB,
-            const SubInfo* __restrict__ subs, const int64_t* __restrict__ tile_row0,
-            const float* __restrict__ piv, const double* __restrict__ rin, const double* __restrict__ qin,
-            const CgScalars* __restrict__ csc, float* __restrict__ zf, const TP* __restrict__ psi,
-            float* __restrict__ rc, int ld, int cmax, int depth, int64_t budget, SolveState* st, int32_t* err,
-            int probe) {
-    pdl_wait();
-    if (st != nullptr && st->done) return;
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
-    // 1024-byte aligned tile ring, then mbarriers, y/x ring, scratch
-    unsigned char* base = smem_align1024(smem_raw);
-    const SubInfo S = subs[blockIdx.x];
-    if (!AMS_ROW_OK(S.row0, 5) || !AMS_ROW_OK(S.row0 + S.n - 1, 5)) return;
-    const int c = S.c, nb = S.nb, n = S.n;
-    const int D = depth;
-    const int nbuf = cmax + D + 1;
-    float* tiles = (float*)base;                                        // nbuf * cmax * 1024
-    uint64_t* bars = (uint64_t*)(tiles + (size_t)nbuf * cmax * 1024);    // ring_bar_slots(nbuf)
-    // y/x ring and scratch: rows of lds = ld + 4 floats, so that the 32 lanes
-    // storing their own rows hit distinct banks (a row stride of ld floats
-    // put every lane on the same bank) while rows stay 16-byte aligned
-    const int lds = local_tma_row_stride(ld);
-    float* ring = (float*)(bars + ring_bar_slots(nbuf));                 // (cmax+1)*32*lds
-    float* tmp = ring + (size_t)(cmax + 1) * 32 * lds;                   // 32*lds
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int rhs0 = warp * NR;
-    const int m = S.m;
-    const int64_t trow = tile_row0[blockIdx.x];      // first tensor row of this subdomain
-    const uint32_t tile_bytes = 4096u * (uint32_t)c;
-    // Per slot: the parity of its next completion, and whether a copy was
-    // issued into it and not yet seen complete.  Both change only when a
-    // wait succeeds, so after a wait runs out the exit drain still waits
-    // for that slot's copy at the parity it was issued with.  Every thread
-    // keeps its own copy (issue and wait are called by all threads).
-    uint32_t phase = 0, pend = 0;
-    bool ok = true;
-
-    if (threadIdx.x == 0) {
-        for (int i = 0; i <= nbuf; ++i) mbar_init(smem_u32(bars + i), 1);
-        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-    }
-    __syncthreads();
-
-    auto issue = [&](const CUtensorMap* map, int K) {
-        if (threadIdx.x == 0) {
-            const int slot = K % nbuf;
-            const uint32_t bar = smem_u32(bars + slot);
-            mbar_expect_tx(bar, tile_bytes);
-            for (int d = 0; d < c; ++d)
-                tma_load_2d(smem_u32(tiles + ((size_t)slot * cmax + d) * 1024), map, 0,
-                            (int32_t)(trow + ((int64_t)K * c + d) * 32), bar);
-        }
-        pend |= 1u << (K % nbuf);
-    };
-    auto wait_slot = [&](int K) {
-        const int slot = K % nbuf;
-        const uint32_t par = (phase >> slot) & 1u;
-        if (!mbar_wait(smem_u32(bars + slot), par, budget)) {
-            ok = false;
-            return;
-        }
-        phase ^= 1u << slot;
-        pend &= ~(1u << slot);
-    };
-    auto slot_tile = [&](int K, int d) -> const float* {
-        return tiles + ((size_t)(K % nbuf) * cmax + d) * 1024;
-    };
-
-    float racc[MM][NR];
-#pragma unroll
-    for (int k = 0; k < MM; ++k)
-#pragma unroll
-        for (int j = 0; j < NR; ++j) racc[k][j] = 0.f;
-
-    // Per-row inputs of block row K (r, basis row, pivot; y in the backward
-    // sweep) sit in PF rotating register buffers: the step that consumes
-    // buffer u reloads it with row K+PF (forward) or K-PF (backward), so
-    // every global load has PF steps to arrive.  The step loop is unrolled
-    // by PF so that buffer indices are compile-time constants.
-    constexpr int PF = (NR <= 2) ? 4 : 2;
-    // Loaded values stay in their loaded type until use (see the
-    // one-right-hand-side kernel below).
-    // r' = r - alpha q for (system, rhs) pairs still iterating
-    double al[NR];
-    bool upd[NR];
-#pragma unroll
-    for (int j = 0; j < NR; ++j) {
-        al[j] = 0.0;
-        upd[j] = false;
-        if (qin != nullptr) {
-            const CgScalars cj = csc[(int64_t)S.seg * ld + rhs0 + j];
-            upd[j] = cj.active != 0;
-            if (upd[j]) al[j] = cj.rho / cj.pq;
-        }
-    }
-    double bt[PF][NR], bq[PF][NR];
-    TP bp[PF][MM];
-    float bv[PF];
-    auto load_fwd = [&](int K, double (&tv)[NR], double (&qv)[NR], TP (&pv)[MM], float& pvt) {
-        const int row = K * 32 + lane;
-        const bool valid = K < nb && row < n;
-        const int64_t grow = S.row0 + row;
-        pvt = 1.f;
-#pragma unroll
-        for (int j = 0; j < NR; ++j) {
-            tv[j] = 0.0;
-            qv[j] = 0.0;
-        }
-#pragma unroll
-        for (int k = 0; k < MM; ++k) pv[k] = TP(0.f);
-        if (valid) {
-            pvt = piv[grow];
-#pragma unroll
-            for (int j = 0; j < NR; ++j) {
-                tv[j] = rin[grow * ld + rhs0 + j];
-                if (upd[j]) qv[j] = qin[grow * ld + rhs0 + j];
-            }
-            if (rc != nullptr) {
-#pragma unroll
-                for (int k = 0; k < MM; ++k)
-                    if (k < m) pv[k] = psi[S.psi_off + (int64_t)row * m + k];
-            }
-        }
-    };
-#pragma unroll
-    for (int u = 0; u < PF; ++u) load_fwd(u, bt[u], bq[u], bp[u], bv[u]);
-
-    auto fwd_step = [&](int K, double (&tb)[NR], double (&qb)[NR], TP (&pb)[MM], float& vb) {
-        if (K + D < nb) issue(&tmF, K + D);
-        float t[NR], pv[MM];
-        const float pvt = vb;
-#pragma unroll
-        for (int j = 0; j < NR; ++j) t[j] = f64_to_f32(upd[j] ? fma(-al[j], qb[j], tb[j]) : tb[j]);
-#pragma unroll
-        for (int k = 0; k < MM; ++k) pv[k] = to_f(pb[k]);
-        load_fwd(K + PF, tb, qb, pb, vb);
-        wait_slot(K);
-        ok = __syncthreads_and(ok);      // uniform decision across the block
-        if (!ok) return;
-        const int row = K * 32 + lane;
-        const bool valid = row < n;
-        const int64_t grow = S.row0 + row;
-        if (rc != nullptr) {
-#pragma unroll
-            for (int k = 0; k < MM; ++k)
-#pragma unroll
-                for (int j = 0; j < NR; ++j) racc[k][j] += pv[k] * t[j];
-        }
-        for (int d = 0; d < c; ++d) {
-            const int src = K - c + d;
-            if (src < 0) continue;
-            const float* ys = ring + (size_t)(src % (c + 1)) * 32 * lds;
-            if (d == 0) tile_rowdot<NR, 1>(slot_tile(K, d), lane, ys, lds, rhs0, -1.f, t);
-            else tile_rowdot<NR, 0>(slot_tile(K, d), lane, ys, lds, rhs0, -1.f, t);
-        }
-        store_row<NR>(tmp + lane * lds + rhs0, t);
-        __syncwarp();
-        float y[NR];
-#pragma unroll
-        for (int j = 0; j < NR; ++j) y[j] = pvt * t[j];
-        tile_rowdot<NR, 2>(slot_tile(K, 0), lane, tmp, lds, rhs0, 1.f, y);
-        float* yr = ring + (size_t)(K % (c + 1)) * 32 * lds;
-        store_row<NR>(yr + lane * lds + rhs0, y);
-        if (valid) {
-#pragma unroll
-            for (int j = 0; j < NR; ++j) zf[grow * ld + rhs0 + j] = y[j];
-        }
-        __syncthreads();
-    };
-
-    // ---------------- forward ----------------
-    for (int j = 0; j < D && j < nb; ++j) issue(&tmF, j);
-    if (probe) {   // timeout test hook: a bounded wait on a barrier nothing completes
-        if (!mbar_wait(smem_u32(bars + nbuf), 0u, budget)) ok = false;
-        ok = __syncthreads_and(ok);
-    }
-#pragma unroll 1
-    for (int K0 = 0; K0 < nb && ok; K0 += PF) {
-#pragma unroll
-        for (int u = 0; u < PF; ++u)
-            if (K0 + u < nb && ok) fwd_step(K0 + u, bt[u], bq[u], bp[u], bv[u]);
-    }
-    if (rc != nullptr && ok) {
-#pragma unroll
-        for (int k = 0; k < MM; ++k)
-#pragma unroll
-            for (int j = 0; j < NR; ++j) {
-                float v = racc[k][j];
-                for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-                if (lane == 0 && k < m) rc[(S.coff + k) * ld + rhs0 + j] = v;
-            }
-    }
-    pdl_trigger();
-    // ---------------- backward ----------------
-    float bw[PF][NR];
-    auto load_bwd = [&](int K, float (&wv)[NR], float& pvt) {
-        const int row = K * 32 + lane;
-        const bool valid = K >= 0 && row < n;
-        const int64_t grow = S.row0 + row;
-        pvt = 1.f;
-#pragma unroll
-        for (int j = 0; j < NR; ++j) wv[j] = 0.f;
-        if (valid) {
-            pvt = piv[grow];
-#pragma unroll
-            for (int j = 0; j < NR; ++j) wv[j] = zf[grow * ld + rhs0 + j];
-        }
-    };
-    auto bwd_step = [&](int K, float (&wb)[NR], float& vb) {
-        if (K - D >= 0) issue(&tmB, K - D);
-        float w[NR];
-        const float pvt = vb;
-#pragma unroll
-        for (int j = 0; j < NR; ++j) w[j] = wb[j];
-        load_bwd(K - PF, wb, vb);
-        wait_slot(K);
-        ok = __syncthreads_and(ok);
-        if (!ok) return;
-        const int row = K * 32 + lane;
-        const bool valid = row < n;
-        const int64_t grow = S.row0 + row;
-        for (int d = 1; d <= c; ++d) {
-            const int src = K + d;
-            if (src >= nb) break;
-            const float* xs = ring + (size_t)(src % (c + 1)) * 32 * lds;
-            // transposed tile of L_{K+d,K}: dense tile c-d of block row K+d,
-            // or (d == c) the upper part of M_{K+c} (rows r <= lane of M^T)
-            if (d < c) tile_rowdot<NR, 0>(slot_tile(src, c - d), lane, xs, lds, rhs0, -1.f, w);
-            else tile_rowdot<NR, 3>(slot_tile(src, 0), lane, xs, lds, rhs0, -1.f, w);
-        }
-        store_row<NR>(tmp + lane * lds + rhs0, w);
-        __syncwarp();
-        float x[NR];
-#pragma unroll
-        for (int j = 0; j < NR; ++j) x[j] = pvt * w[j];
-        // L_KK^{-T}: strict lower part of M_K read as row `lane` of M_K^T (r > lane)
-        tile_rowdot<NR, 4>(slot_tile(K, 0), lane, tmp, lds, rhs0, 1.f, x);
-        float* xr = ring + (size_t)(K % (c + 1)) * 32 * lds;
-        store_row<NR>(xr + lane * lds + rhs0, x);
-        if (valid) {
-#pragma unroll
-            for (int j = 0; j < NR; ++j) zf[grow * ld + rhs0 + j] = x[j];
-        }
-        __syncthreads();
-    };
-    if (ok) {
-#pragma unroll
-        for (int u = 0; u < PF; ++u) load_bwd(nb - 1 - u, bw[u], bv[u]);
-        for (int j = 0; j < D && nb - 1 - j >= 0; ++j) issue(&tmB, nb - 1 - j);
-    }
-#pragma unroll 1
-    for (int K0 = nb - 1; K0 >= 0 && ok; K0 -= PF) {
-#pragma unroll
-        for (int u = 0; u < PF; ++u)
-            if (K0 - u >= 0 && ok) bwd_step(K0 - u, bw[u], bv[u]);
-    }
-    if (!ok) timeout_drain(bars, nbuf, pend, phase, err, st, threadIdx.x == 0);
-}
-
 
 // ---------------------------------------------------------------------------
 // One right-hand side: one warp per subdomain, forward tiles only.
@@ -398,37 +48,6 @@ k_local_tma(const __grid_constant__ CUtensorMap tmF, const __grid_constant__ CUt
 //     chunk that holds the diagonal), and each 32-term dot is summed as a
 //     tree of eight 4-term dots.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ float dot4(const float4& a, const float4& b) {
-    return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, a.x * b.x)));
-}
-__device__ __forceinline__ float4 mul4(const float4& a, const float4& b) {
-    return make_float4(a.x * b.x, a.y * b.y, a.z * b.z, a.w * b.w);
-}
-__device__ __forceinline__ float sum8(const float (&c)[8]) {
-    return ((c[0] + c[1]) + (c[2] + c[3])) + ((c[4] + c[5]) + (c[6] + c[7]));
-}
-__device__ __forceinline__ float wsum8(const float (&w)[8], const float (&c)[8]) {
-    const float a = fmaf(w[1], c[1], w[0] * c[0]);
-    const float b = fmaf(w[3], c[3], w[2] * c[2]);
-    const float d = fmaf(w[5], c[5], w[4] * c[4]);
-    const float e = fmaf(w[7], c[7], w[6] * c[6]);
-    return (a + b) + (d + e);
-}
-// Column `lane` of a swizzled tile against a broadcast vector v[0..31]:
-// c[j] = sum_{r in chunk j} T[r][lane] v[r].
-__device__ __forceinline__ void col_chunks(const float* T, const int (&csw)[8], const float* v, float (&c)[8]) {
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const float4 x = *reinterpret_cast<const float4*>(v + 4 * j);
-        const int r = 4 * j;
-        const float a0 = T[(r + 0) * 32 + csw[(r + 0) & 7]];
-        const float a1 = T[(r + 1) * 32 + csw[(r + 1) & 7]];
-        const float a2 = T[(r + 2) * 32 + csw[(r + 2) & 7]];
-        const float a3 = T[(r + 3) * 32 + csw[(r + 3) & 7]];
-        c[j] = fmaf(a3, x.w, fmaf(a2, x.z, fmaf(a1, x.y, a0 * x.x)));
-    }
-}
-
 // Packed FP32 pairs (FFMA2, sm_100 and later): a 32-term dot product in
 // 16 two-wide fused multiply-adds on four independent accumulators.
 __device__ __forceinline__ float2 lo2(const float4& v) { return make_float2(v.x, v.y); }
@@ -521,7 +140,7 @@ k_local_tma1(const __grid_constant__ CUtensorMap tmF, const SubInfo* __restrict_
     const uint32_t tile_bytes = 4096u * (uint32_t)c;
     const int slot_floats = cmax * 1024;
     // parity of each slot's next completion, and the slots with a copy in
-    // flight; both change only when a wait succeeds (see k_local_tma)
+    // flight; both change only when a wait succeeds, so the exit drain waits for every copy
     uint32_t phase = 0, pend = 0;
     bool ok = true;
 
@@ -634,7 +253,7 @@ k_local_tma1(const __grid_constant__ CUtensorMap tmF, const SubInfo* __restrict_
     if (qin != nullptr) {
         const CgScalars cs = csc[S.seg];
         upd = cs.active != 0;
-        if (upd) alpha = cs.rho / cs.pq;
+        if (upd) alpha = cs.alpha;
     }
     const double* rp = rin + S.row0 + lane;
     const double* qp = upd ? qin + S.row0 + lane : nullptr;
@@ -807,63 +426,6 @@ k_local_tma1(const __grid_constant__ CUtensorMap tmF, const SubInfo* __restrict_
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-size_t local_tma_smem(int cmax, int ld, int depth) {
-    const int nbuf = cmax + depth + 1;
-    const int lds = local_tma_row_stride(ld);
-    return 1024 /* alignment slack */ + (size_t)nbuf * cmax * 4096 + (size_t)ring_bar_slots(nbuf) * 8 +
-           ((size_t)(cmax + 1) * 32 * lds + 32 * lds) * sizeof(float);
-}
-
-// Prefetch depth: block rows in flight per subdomain.  Deeper rings hide
-// more TMA latency but cost shared memory; the single-warp blocks of the
-// one-right-hand-side case must stay small enough for about eight resident
-// blocks per SM.
-int local_tma_depth(int cmax, int ld) {
-    const size_t budget = (ld == 1) ? 32 * 1024 : 100 * 1024;
-    int d = 6;
-    while (d > 1 && local_tma_smem(cmax, ld, d) > budget) --d;
-    return d;
-}
-
-template <typename TP, int NR, int MM>
-static cudaError_t tma_nr(const LocalTmaArgs& a, const void* psi, void* zf, void* rc) {
-    const int warps = a.ld / NR;
-    const int depth = a.depth > 0 ? a.depth : local_tma_depth(a.cmax, a.ld);
-    const size_t smem = local_tma_smem(a.cmax, a.ld, depth);
-    auto kern = k_local_tma<TP, NR, MM>;
-    static size_t smem_set = 0;
-    if (smem > smem_set) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        smem_set = smem;
-    }
-    return launch_kernel(a.pdl, kern, dim3(a.nsub), dim3(warps * 32), smem, a.stream, *a.tmF, *a.tmB, a.subs,
-                         a.tile_row0, a.piv, a.in.r, a.in.q, a.in.sc, (float*)zf, (const TP*)psi, (float*)rc, a.ld,
-                         a.cmax, depth, a.budget, a.st, a.err, a.probe);
-}
-
-template <typename TP>
-static cudaError_t tma_tp(const LocalTmaArgs& a, const void* psi, void* zf, void* rc) {
-    const bool big = a.mmax > 8;
-    const int nrmax = big ? 4 : 8;
-    int nr = a.ld < nrmax ? a.ld : nrmax;
-    // fewer right-hand sides per warp: more warps per block (at most 8, the kernel's launch bound)
-    if (a.nr > 0 && a.nr < nr && a.ld / a.nr <= 8) nr = a.nr;
-    if (big) {
-        switch (nr) {
-            case 1: return tma_nr<TP, 1, 16>(a, psi, zf, rc);
-            case 2: return tma_nr<TP, 2, 16>(a, psi, zf, rc);
-            default: return tma_nr<TP, 4, 16>(a, psi, zf, rc);
-        }
-    }
-    switch (nr) {
-        case 1: return tma_nr<TP, 1, 8>(a, psi, zf, rc);
-        case 2: return tma_nr<TP, 2, 8>(a, psi, zf, rc);
-        case 4: return tma_nr<TP, 4, 8>(a, psi, zf, rc);
-        default: return tma_nr<TP, 8, 8>(a, psi, zf, rc);
-    }
-}
-
 size_t local_tma1_smem(int cmax, int nbmax, int depth) {
     const int nbuf = cmax + depth + 1;
     return 1024 /* alignment slack */ + (size_t)nbuf * cmax * 4096 + (size_t)ring_bar_slots(nbuf) * 8 +
@@ -896,31 +458,28 @@ static cudaError_t tma1(const LocalTmaArgs& a, const void* psi, void* zf, void* 
 }
 
 // The one-right-hand-side kernel keeps y for a whole subdomain in shared
-// memory; wider subdomains use the general kernel.
+// memory; larger subdomains and more right-hand sides use the MMA kernel.
+// (At 3 right-hand sides, 96x80x72 cells in 8^3 blocks, a row-per-lane FP32
+// kernel took 152 us a launch, the MMA kernel with five of its eight
+// columns empty 117 us.)
 static bool use_tma1(const LocalTmaArgs& a) {
     return a.ld == 1 && local_tma1_smem(a.cmax, a.nbmax, 2) <= 200 * 1024;
 }
 
 size_t local_tma_launch_smem(const LocalTmaArgs& a, int depth) {
-    if (use_tma1(a)) return local_tma1_smem(a.cmax, a.nbmax, depth);
-    return a.ld >= 8 ? local_mma_smem(a.cmax, a.ld, depth) : local_tma_smem(a.cmax, a.ld, depth);
+    return use_tma1(a) ? local_tma1_smem(a.cmax, a.nbmax, depth) : local_mma_smem(a.cmax, a.ld, depth);
 }
 
-cudaError_t launch_local_tma(const LocalTmaArgs& a, int prec, const void* psi, void* zf, void* rc) {
-    // 8 or more right-hand sides: the tile products on the tensor cores
-    if (!use_tma1(a) && a.ld >= 8) return launch_local_mma(a, prec, psi, zf, rc);
-    if (use_tma1(a)) {
-        const bool big = a.mmax > 8, c1 = a.cmax == 1;
-        if (prec == AMS_PREC_FP32) {
-            if (big) return c1 ? tma1<float, 16, true>(a, psi, zf, rc) : tma1<float, 16, false>(a, psi, zf, rc);
-            return c1 ? tma1<float, 8, true>(a, psi, zf, rc) : tma1<float, 8, false>(a, psi, zf, rc);
-        }
-        if (big)
-            return c1 ? tma1<__nv_bfloat16, 16, true>(a, psi, zf, rc) : tma1<__nv_bfloat16, 16, false>(a, psi, zf, rc);
-        return c1 ? tma1<__nv_bfloat16, 8, true>(a, psi, zf, rc) : tma1<__nv_bfloat16, 8, false>(a, psi, zf, rc);
+cudaError_t launch_local_tma(const LocalTmaArgs& a, int prec, const void* psi, const void* psif, void* zf, void* rc) {
+    if (!use_tma1(a)) return launch_local_mma(a, prec, psif, zf, rc);
+    const bool big = a.mmax > 8, c1 = a.cmax == 1;
+    if (prec == AMS_PREC_FP32) {
+        if (big) return c1 ? tma1<float, 16, true>(a, psi, zf, rc) : tma1<float, 16, false>(a, psi, zf, rc);
+        return c1 ? tma1<float, 8, true>(a, psi, zf, rc) : tma1<float, 8, false>(a, psi, zf, rc);
     }
-    if (prec == AMS_PREC_FP32) return tma_tp<float>(a, psi, zf, rc);
-    return tma_tp<__nv_bfloat16>(a, psi, zf, rc);
+    if (big)
+        return c1 ? tma1<__nv_bfloat16, 16, true>(a, psi, zf, rc) : tma1<__nv_bfloat16, 16, false>(a, psi, zf, rc);
+    return c1 ? tma1<__nv_bfloat16, 8, true>(a, psi, zf, rc) : tma1<__nv_bfloat16, 8, false>(a, psi, zf, rc);
 }
 
 // 2-D view [rows x 32] FP32 of a tile array; one box = one 32x32 tile,

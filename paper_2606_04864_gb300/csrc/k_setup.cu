@@ -149,13 +149,13 @@ __global__ void k_band_pack(const SubInfo* __restrict__ subs, const int64_t* __r
     }
 }
 
-// Same factor, TMA tile layout: forward tiles row-major, backward tiles
-// transposed, reciprocal pivots per row (FP32).  One warp per (subdomain,
-// block row); lane = tile column.
+// Same factor as FP32 tiles, row-major (one-RHS kernel) and in MMA fragment
+// order (several), and the reciprocal pivots per row.  One warp per
+// (subdomain, block row); lane = tile column.
 __global__ void k_band_pack_tiles(const SubInfo* __restrict__ subs, const int64_t* __restrict__ band_off,
                                   const int2* __restrict__ work, const double* __restrict__ band,
                                   const int64_t* __restrict__ out_off, float* __restrict__ fwd,
-                                  float* __restrict__ bwd, float* __restrict__ piv) {
+                                  float* __restrict__ mma, float* __restrict__ piv) {
     const int2 wk = work[blockIdx.x];
     const int s = wk.x, K = wk.y;
     const SubInfo Sb = subs[s];
@@ -181,14 +181,14 @@ __global__ void k_band_pack_tiles(const SubInfo* __restrict__ subs, const int64_
     for (int r = 0; r < 32; ++r) {
         const float v = (float)(lane >= r ? Lval(r0 + r, cb + lane) : x[r]);
         fwd[tbase + r * 32 + lane] = v;
-        bwd[tbase + lane * 32 + r] = v;
+        mma[tbase + mma_tile_off(r, lane)] = v;
     }
     for (int t = 1; t < c; ++t) {
         const int64_t cbt = 32LL * (K - c + t);
         for (int r = 0; r < 32; ++r) {
             const float v = (float)Lval(r0 + r, cbt + lane);
             fwd[tbase + (int64_t)t * 1024 + r * 32 + lane] = v;
-            bwd[tbase + (int64_t)t * 1024 + lane * 32 + r] = v;
+            mma[tbase + (int64_t)t * 1024 + mma_tile_off(r, lane)] = v;
         }
     }
     const int64_t row = r0 + lane;
@@ -712,9 +712,9 @@ void launch_band_pack_work(cudaStream_t s, int nwork, const SubInfo* subs, const
     k_band_pack<<<nwork, 32, 0, s>>>(subs, band_off, work, band, out_off, out64, out32);
 }
 void launch_band_pack_tiles(cudaStream_t s, int nwork, const SubInfo* subs, const int64_t* band_off,
-                            const int2* work, const double* band, const int64_t* out_off, float* fwd, float* bwd,
+                            const int2* work, const double* band, const int64_t* out_off, float* fwd, float* mma,
                             float* piv) {
-    k_band_pack_tiles<<<nwork, 32, 0, s>>>(subs, band_off, work, band, out_off, fwd, bwd, piv);
+    k_band_pack_tiles<<<nwork, 32, 0, s>>>(subs, band_off, work, band, out_off, fwd, mma, piv);
 }
 void launch_eig_init(cudaStream_t s, int nsub, const SubInfo* subs, int P, double* X) {
     k_eig_init<<<nsub, 256, 0, s>>>(subs, P, X);

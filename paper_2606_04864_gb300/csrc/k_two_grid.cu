@@ -48,7 +48,7 @@ k_tg_resid(const int64_t* __restrict__ sell_ptr, const int32_t* __restrict__ sel
     if (q != nullptr) {
         const CgScalars c = sc[(int64_t)R.blk_seg[blockIdx.x] * LD + rhs];
         upd = c.active != 0;
-        if (upd) alpha = c.rho / c.pq;
+        if (upd) alpha = c.alpha;
     }
     const int64_t lo = R.blk_lo[blockIdx.x], hi = R.blk_lo[blockIdx.x + 1];
     for (int64_t e = lo + threadIdx.x; e < hi; e += kRedThreads) {

@@ -77,8 +77,10 @@ struct LocalTmaArgs {
     int nsub;
     const SubInfo* subs;
     const struct CUtensorMap_st* tmF;
-    const struct CUtensorMap_st* tmB;
     const int64_t* tile_row0;
+    const float* mma_tiles;  // the tiles in MMA fragment order, and the first element of each subdomain's
+    const int64_t* mma_off;
+    const int64_t* brow0;    // block rows of the subdomains before each
     const float* piv;
     ResidIn in;
     int ld;
@@ -89,7 +91,7 @@ struct LocalTmaArgs {
     SolveState* st;
     bool pdl;
     int depth;               // ring depth (block rows in flight); 0: chosen from the band width
-    int nr;                  // several-RHS kernel: right-hand sides per warp (1, 2, 4, 8); 0: default
+    int nr;                  // several-RHS kernel: right-hand sides per warp (8, or 16 from 16 on); else default
     int l2mode;              // one-RHS kernel, L2 priority of factor tiles: 0 none, 1 evict-first on
                              // tiles read for the last time, 2 as 1 plus evict-last on kept tiles
     int l2keep;              // block rows below the ring's resident ones whose forward load is
@@ -132,16 +134,20 @@ int local_solve_depth(int cmax, int ld, size_t tf_bytes);
 cudaError_t launch_local_solve(const LocalSolveArgs& a, int prec, const void* fac, const void* psi,
                                void* zf, void* rc);
 void launch_coarse_gemm(const CoarseLaunch& c, int prec, int ld, const void* in, void* out);
-cudaError_t launch_local_tma(const LocalTmaArgs& a, int prec, const void* psi, void* zf, void* rc);
-// 8 to 32 right-hand sides: tile products as tensor-core MMAs (k_local_mma.cu)
-cudaError_t launch_local_mma(const LocalTmaArgs& a, int prec, const void* psi, void* zf, void* rc);
+// psif: the basis in fragment order (launch_pack_psi), read by the MMA kernel
+cudaError_t launch_local_tma(const LocalTmaArgs& a, int prec, const void* psi, const void* psif, void* zf, void* rc);
+// several right-hand sides: tile products as tensor-core MMAs (k_local_mma.cu)
+cudaError_t launch_local_mma(const LocalTmaArgs& a, int prec, const void* psif, void* zf, void* rc);
 size_t local_mma_smem(int cmax, int ld, int depth);
-size_t local_tma_smem(int cmax, int ld, int depth);
+// Basis in MMA fragment order: 16-byte words per block row, and the packing
+size_t local_mma_psi_words(int prec, int mmax);
+void launch_pack_psi(cudaStream_t s, int nsub, const SubInfo* subs, const int64_t* brow0, int prec, int mmax,
+                     const void* psi, void* out);
 // Shared memory the TMA local-solve launch for `a` needs at ring depth `depth`.
 size_t local_tma_launch_smem(const LocalTmaArgs& a, int depth);
 cudaError_t make_tile_map(void* base, int64_t rows, struct CUtensorMap_st* out);
 void launch_band_pack_tiles(cudaStream_t s, int nwork, const SubInfo* subs, const int64_t* band_off,
-                            const int2* work, const double* band, const int64_t* out_off, float* fwd, float* bwd,
+                            const int2* work, const double* band, const int64_t* out_off, float* fwd, float* mma,
                             float* piv);
 struct ProlongArgs {
     const void* psi;
