@@ -110,7 +110,7 @@ struct ams_handle_s {
     cudaStream_t stream = nullptr;      // internal non-blocking stream (all device work)
     cudaStream_t ustream = nullptr;     // caller's stream (ordering only)
     cudaEvent_t ev_enter = nullptr;
-    std::map<int, cudaGraphExec_t> loop_graph;   // device-resident iteration loop per ld
+    std::map<int, cudaGraphExec_t> loop_graph;   // device-resident iteration loop per loop_key
     KernelProfile* prof = nullptr;
     int prec = AMS_PREC_FP32_BF16;
     int flexible = 1;
@@ -164,6 +164,7 @@ struct ams_handle_s {
     int32_t* d_cnt = nullptr;
     // solve work space (sized for ld_alloc)
     int ld_alloc = 0, ld_last = 0;
+    int ncols = 1;              // right-hand sides of the current call
     double *d_x = nullptr, *d_r = nullptr, *d_p = nullptr, *d_q = nullptr, *d_z = nullptr;
     double* d_p2 = nullptr;             // second direction buffer (iterations alternate p and p2)
     void *d_zf = nullptr, *d_rc = nullptr, *d_yc = nullptr, *d_ec = nullptr;
@@ -555,7 +556,7 @@ static ams_status setup_eigen(ams_handle h, const int64_t* d_rowptr, const int32
     SubInfo* d_esubs = nullptr;
     AMS_TRY(upload(h, &d_esubs, esubs));
     LocalSolveArgs la{h->stream, h->N, d_esubs, ResidIn{d_X, nullptr, nullptr}, d_S, P, h->cmax, 0, nullptr, false,
-                      0};
+                      0, P};
     const int maxit = h->opt.eig_maxit > 0 ? h->opt.eig_maxit : 300;
     const double tol = h->opt.eig_tol > 0 ? h->opt.eig_tol : 1e-13;
     std::vector<double> res(h->N);
@@ -563,7 +564,7 @@ static ams_status setup_eigen(ams_handle h, const int64_t* d_rowptr, const int32
     double worst = 0.0;
     const int ncheck = std::min(P, mreq + 1);
     for (it = 1; it <= maxit; ++it) {
-        AMS_CUDA_TRY(launch_local_solve(la, AMS_PREC_FP64, d_efac, nullptr, d_Y, nullptr));
+        AMS_CUDA_TRY(launch_local_solve(la, (const double*)d_efac, nullptr, d_Y, nullptr));
         // Rayleigh-Ritz on the iterations whose residuals are checked; on the
         // others only the S-orthonormalisation (the span is the same)
         const bool check = it % 4 == 0 || it == maxit;
@@ -1328,8 +1329,9 @@ static ams_status launch_local(ams_handle h, int ld, const ResidIn& in, bool wit
         AMS_CUDA_TRY(launch_local_tma(a, h->prec, h->d_psi, h->d_psif, h->d_zf, coarse ? h->d_rc : nullptr));
     } else {
         LocalSolveArgs la{h->stream, h->N, h->d_subs, in, nullptr, ld, h->cmax, std::max(1, h->mmax),
-                          with_state ? h->d_st : nullptr, h->use_pdl, h->tune[ld].depth};
-        AMS_CUDA_TRY(launch_local_solve(la, h->prec, h->d_fac, h->d_psi, h->d_zf, coarse ? h->d_rc : nullptr));
+                          with_state ? h->d_st : nullptr, h->use_pdl, h->tune[ld].depth, h->ncols};
+        AMS_CUDA_TRY(launch_local_solve(la, (const double*)h->d_fac, (const double*)h->d_psi, (double*)h->d_zf,
+                                        coarse ? (double*)h->d_rc : nullptr));
     }
     return AMS_OK;
 }
@@ -1346,6 +1348,7 @@ constexpr int kPowerSteps = 300;
 
 static ams_status estimate_two_grid_omega(ams_handle h) {
     const double c = -h->opt.two_grid_omega;
+    h->ncols = 1;
     AMS_TRY(ensure_work(h, 1));
     RedCache *rc = nullptr, *rcs = nullptr;
     AMS_TRY(get_red(h, 1, &rc, &rcs));
@@ -1555,8 +1558,13 @@ static ams_status launch_iteration(ams_handle h, const LaunchCtx& L, int par) {
 // device timeout) or after `cap` bodies.  Kernel arguments are fixed device
 // pointers and every scalar lives in device memory, so one graph launch
 // runs the solve to the end with no host round trip.
+// The FP64 local solves are launched for the call's right-hand sides, the
+// other kernels for their power of two ld: one graph per number that matters.
+static int loop_key(ams_handle h, int ld) { return h->prec == AMS_PREC_FP64 ? h->ncols : ld; }
+
 static ams_status get_loop_graph(ams_handle h, const LaunchCtx& L, cudaGraphExec_t* out) {
-    auto it = h->loop_graph.find(L.ld);
+    const int key = loop_key(h, L.ld);
+    auto it = h->loop_graph.find(key);
     if (it != h->loop_graph.end()) {
         *out = it->second;
         return AMS_OK;
@@ -1591,7 +1599,7 @@ static ams_status get_loop_graph(ams_handle h, const LaunchCtx& L, cudaGraphExec
     AMS_CUDA_TRY(e);
     cudaGraphExec_t ex = nullptr;
     AMS_CUDA_TRY(cudaGraphInstantiate(&ex, g, 0));
-    h->loop_graph[L.ld] = ex;
+    h->loop_graph[key] = ex;
     *out = ex;
     return AMS_OK;
 }
@@ -1819,6 +1827,7 @@ static ams_status autotune(ams_handle h, const double* f_dev, int nrhs, int ld) 
 static ams_status pcg_launch(ams_handle h, const double* f_dev, int nrhs, double rtol, double* u_dev,
                              const double* u0_dev = nullptr) {
     const int ld = pow2ceil(nrhs);
+    h->ncols = nrhs;
     AMS_TRY(ensure_work(h, ld));
     RedCache *rc = nullptr, *rcs = nullptr;
     AMS_TRY(get_red(h, ld, &rc, &rcs));
@@ -2242,11 +2251,13 @@ ams_status ams_set_launch_shape(ams_handle h, int32_t nrhs, const int32_t* shape
     T.depth = depth;
     T.nr = nr;
     T.done = true;
-    auto g = h->loop_graph.find(ld);   // captured with the previous shapes
-    if (g != h->loop_graph.end()) {
-        AMS_CUDA_TRY(cudaGraphExecDestroy(g->second));
-        h->loop_graph.erase(g);
-    }
+    for (auto g = h->loop_graph.begin(); g != h->loop_graph.end();)   // captured with the previous shapes
+        if (pow2ceil(g->first) == ld) {
+            AMS_CUDA_TRY(cudaGraphExecDestroy(g->second));
+            g = h->loop_graph.erase(g);
+        } else {
+            ++g;
+        }
     return AMS_OK;
 }
 
@@ -2352,6 +2363,7 @@ ams_status ams_apply_preconditioner(ams_handle h, const double* r, int32_t nrhs,
         return AMS_ERR_INVALID_ARG;
     }
     const int ld = pow2ceil(nrhs);
+    h->ncols = nrhs;
     AMS_TRY(ensure_work(h, ld));
     RedCache *rc = nullptr, *rcs = nullptr;
     AMS_TRY(get_red(h, ld, &rc, &rcs));
@@ -2412,6 +2424,7 @@ ams_status ams_time_kernel(ams_handle h, int32_t which, int32_t reps, double* av
     }
     AMS_TRY(enter(h));
     const int ld = h->ld_last;
+    h->ncols = ld;
     RedCache *rc = nullptr, *rcs = nullptr;
     AMS_TRY(get_red(h, ld, &rc, &rcs));
     LaunchCtx L = make_ctx(h, *rc, *rcs);

@@ -3,8 +3,8 @@
 // One CG iteration (Section 3.1 preconditioner inside CG) is five kernels:
 //   k_dir_update      p = z + beta p_old
 //   k_spmv_dot        q = A p and p.q                          (SELL-32 SpMV)
-//   k_local_solve     z_f = sum_i R_i^T A_i^{-1} R_i r'  and  r_c = R_0 r',
-//   (k_local_tma*)    r' = r - alpha q formed on the fly       (alpha = rho/pq)
+//   k_local_*         z_f = sum_i R_i^T A_i^{-1} R_i r'  and  r_c = R_0 r',
+//                     r' = r - alpha q formed on the fly       (alpha = rho/pq)
 //   k_coarse_*        y = L_c^{-1} r_c  (k_coarse.cu)          (A_0 = L_c L_c^T)
 //   k_prolong_update  e_c = L_c^{-T} y, z = z_f + R_0^T e_c, r = r',
 //                     x += alpha p, r.z, r.r, z.q, convergence test, beta
@@ -151,263 +151,6 @@ k_x_flush(const double* __restrict__ p, const double* __restrict__ p2, double* _
     const double* pl = ((it - 1) % 2 == 0) ? p2 : p;
     const int64_t lo = R.blk_lo[blockIdx.x], hi = R.blk_lo[blockIdx.x + 1];
     for (int64_t e = lo + threadIdx.x; e < hi; e += kRedThreads) x[e] = fma(alpha, pl[e], x[e]);
-}
-
-// ===========================================================================
-// a3+a4: local solves z_f = A_i^{-1} r_i for every subdomain (one thread
-// block per subdomain, warps split the right-hand sides, NR per warp), with
-// the restriction r_c = Psi_i^T r_i accumulated on the way.
-//
-// Forward sweep over block rows K = 0..nb-1 (lane = row of the block):
-//   t   = r_K - sum_{d<c} L_{K,K-c+d} y_{K-c+d}
-//   y_K = L_KK^{-1} t
-// Backward sweep K = nb-1..0 (lane = column of the block):
-//   w   = y_K - sum_{d=1..c} L_{K+d,K}^T x_{K+d}
-//   x_K = L_KK^{-T} w
-// Factor block rows are staged through shared memory with cp.async in a
-// ring of c+D+1 buffers, D block rows ahead of the sweep (one commit group
-// per block row); y is kept in z_f between the sweeps.
-// ===========================================================================
-template <typename TF, typename TP, int NR, int MM>
-__global__ void k_local_solve(const SubInfo* __restrict__ subs, const TF* __restrict__ fac,
-                              const double* __restrict__ rin, const double* __restrict__ qin,
-                              const CgScalars* __restrict__ csc, const double* __restrict__ rowscale,
-                              TF* __restrict__ zf, const TP* __restrict__ psi, TF* __restrict__ rc,
-                              int ld, int cmax, int depth, const SolveState* st) {
-    pdl_wait();
-    if (st != nullptr && st->done) return;
-    using A = typename Acc<TF>::type;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const SubInfo S = subs[blockIdx.x];
-    const int c = S.c, nb = S.nb, n = S.n;
-    const int D = depth;                                       // block rows in flight
-    const int nbuf = c + D + 1;
-    const int64_t brs = blockrow_elems(c);
-    const int64_t brs_max = blockrow_elems(cmax);
-    TF* bufs = (TF*)smem_raw;                                  // (cmax+D+1) * brs_max
-    TF* ring = bufs + (int64_t)(cmax + D + 1) * brs_max;       // (cmax+1) * 32 * ld
-    TF* tmp = ring + (int64_t)(cmax + 1) * 32 * ld;            // 32 * ld
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    const int rhs0 = warp * NR;
-    const TF* F = fac + S.fac_off;
-    const int m = S.m;
-
-    A racc[MM][NR];
-#pragma unroll
-    for (int k = 0; k < MM; ++k)
-#pragma unroll
-        for (int j = 0; j < NR; ++j) racc[k][j] = A(0);
-
-    // r' = r - alpha q for (system, rhs) pairs still iterating (see ResidIn)
-    double al[NR];
-    bool upd[NR];
-#pragma unroll
-    for (int j = 0; j < NR; ++j) {
-        al[j] = 0.0;
-        upd[j] = false;
-        if (qin != nullptr) {
-            const CgScalars cj = csc[(int64_t)S.seg * ld + rhs0 + j];
-            upd[j] = cj.active != 0;
-            if (upd[j]) al[j] = cj.rho / cj.pq;
-        }
-    }
-    // Inputs of block row K (r and q rows, basis rows, row scale) are
-    // loaded two block rows ahead into alternating register buffers and
-    // kept in their loaded type until the step that uses them, so their
-    // global-memory latency overlaps the substitution of earlier rows.
-    auto load_fwd = [&](int K, double (&rv)[NR], double (&qv)[NR], TP (&pv)[MM], double& scv) {
-        const int row = K * 32 + lane;
-        const bool valid = K < nb && row < n;
-        const int64_t grow = S.row0 + row;
-        scv = 1.0;
-#pragma unroll
-        for (int j = 0; j < NR; ++j) {
-            rv[j] = 0.0;
-            qv[j] = 0.0;
-        }
-#pragma unroll
-        for (int k = 0; k < MM; ++k) pv[k] = TP(0.f);
-        if (valid) {
-            if (rowscale != nullptr) scv = rowscale[grow];
-#pragma unroll
-            for (int j = 0; j < NR; ++j) {
-                rv[j] = rin[grow * ld + rhs0 + j];
-                if (upd[j]) qv[j] = qin[grow * ld + rhs0 + j];
-            }
-            if (rc != nullptr) {
-#pragma unroll
-                for (int k = 0; k < MM; ++k)
-                    if (k < m) pv[k] = psi[S.psi_off + (int64_t)row * m + k];
-            }
-        }
-    };
-    double rb[2][NR], qb[2][NR], sb[2];
-    TP pb[2][MM];
-    load_fwd(0, rb[0], qb[0], pb[0], sb[0]);
-    load_fwd(1, rb[1], qb[1], pb[1], sb[1]);
-
-    // ---------------- forward ----------------
-    // one commit group per block row; row K+D is requested at step K
-    for (int j = 0; j < D; ++j) {
-        if (j < nb) block_copy_async(bufs + (int64_t)(j % nbuf) * brs_max, F + (int64_t)j * brs, brs * sizeof(TF));
-        cp_async_commit();
-    }
-    auto fwd_step = [&](int K, double (&rv)[NR], double (&qv)[NR], TP (&pb_)[MM], double& scv) {
-        if (K + D < nb)
-            block_copy_async(bufs + (int64_t)((K + D) % nbuf) * brs_max, F + (int64_t)(K + D) * brs,
-                             brs * sizeof(TF));
-        cp_async_commit();
-        A t[NR], pv[MM];
-#pragma unroll
-        for (int j = 0; j < NR; ++j) t[j] = (A)((upd[j] ? fma(-al[j], qv[j], rv[j]) : rv[j]) * scv);
-#pragma unroll
-        for (int k = 0; k < MM; ++k) pv[k] = (A)to_d(pb_[k]);
-        load_fwd(K + 2, rv, qv, pb_, scv);
-        cp_async_wait_n(D);
-        __syncthreads();
-        const TF* B = bufs + (int64_t)(K % nbuf) * brs_max;
-        const int row = K * 32 + lane;
-        const bool valid = row < n;
-        const int64_t grow = S.row0 + row;
-        if (rc != nullptr) {
-#pragma unroll
-            for (int k = 0; k < MM; ++k)
-#pragma unroll
-                for (int j = 0; j < NR; ++j) racc[k][j] += pv[k] * t[j];
-        }
-        for (int d = 0; d < c; ++d) {
-            const int src = K - c + d;
-            if (src < 0) continue;
-            const TF* T = B + d * 1024;
-            const TF* ys = ring + (int64_t)(src % (c + 1)) * 32 * ld + rhs0;
-#pragma unroll 8
-            for (int q = 0; q < 32; ++q) {
-                A coef = (A)T[tile_idx(lane, q)];
-                if (d == 0 && q < lane) coef = A(0);
-#pragma unroll
-                for (int j = 0; j < NR; ++j) t[j] -= coef * (A)ys[q * ld + j];
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < NR; ++j) tmp[lane * ld + rhs0 + j] = (TF)t[j];
-        __syncwarp();
-        const A piv = (A)B[c * 1024 + lane];
-        A y[NR];
-#pragma unroll
-        for (int j = 0; j < NR; ++j) y[j] = piv * t[j];
-#pragma unroll 8
-        for (int q = 0; q < 32; ++q) {
-            const A coef = q < lane ? (A)B[tile_idx(lane, q)] : A(0);
-#pragma unroll
-            for (int j = 0; j < NR; ++j) y[j] += coef * (A)tmp[q * ld + rhs0 + j];
-        }
-        TF* yr = ring + (int64_t)(K % (c + 1)) * 32 * ld + rhs0;
-#pragma unroll
-        for (int j = 0; j < NR; ++j) yr[lane * ld + j] = (TF)y[j];
-        if (valid) {
-#pragma unroll
-            for (int j = 0; j < NR; ++j) zf[grow * ld + rhs0 + j] = (TF)y[j];
-        }
-        __syncthreads();
-    };
-#pragma unroll 1
-    for (int K = 0; K < nb; K += 2) {
-        fwd_step(K, rb[0], qb[0], pb[0], sb[0]);
-        if (K + 1 < nb) fwd_step(K + 1, rb[1], qb[1], pb[1], sb[1]);
-    }
-    pdl_trigger();
-    // restriction: reduce over lanes, lane 0 writes r_c rows of this subdomain
-    if (rc != nullptr) {
-#pragma unroll
-        for (int k = 0; k < MM; ++k) {
-#pragma unroll
-            for (int j = 0; j < NR; ++j) {
-                A v = racc[k][j];
-                for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-                if (lane == 0 && k < m) rc[(S.coff + k) * ld + rhs0 + j] = (TF)v;
-            }
-        }
-    }
-    // ---------------- backward ----------------
-    // step K needs block rows K..K+c; row K-D is requested at step K
-    cp_async_wait_all();
-    __syncthreads();
-    for (int j = 0; j < D; ++j) {
-        const int r = nb - 1 - j;
-        if (r >= 0) block_copy_async(bufs + (int64_t)(r % nbuf) * brs_max, F + (int64_t)r * brs, brs * sizeof(TF));
-        cp_async_commit();
-    }
-    auto load_bwd = [&](int K, TF (&wv)[NR]) {
-        const int row = K * 32 + lane;
-        const bool valid = K >= 0 && row < n;
-        const int64_t grow = S.row0 + row;
-#pragma unroll
-        for (int j = 0; j < NR; ++j) wv[j] = TF(0);
-        if (valid) {
-#pragma unroll
-            for (int j = 0; j < NR; ++j) wv[j] = zf[grow * ld + rhs0 + j];
-        }
-    };
-    TF wb[2][NR];
-    load_bwd(nb - 1, wb[0]);
-    load_bwd(nb - 2, wb[1]);
-    auto bwd_step = [&](int K, TF (&wv)[NR]) {
-        if (K - D >= 0)
-            block_copy_async(bufs + (int64_t)((K - D) % nbuf) * brs_max, F + (int64_t)(K - D) * brs,
-                             brs * sizeof(TF));
-        cp_async_commit();
-        A w[NR];
-#pragma unroll
-        for (int j = 0; j < NR; ++j) w[j] = (A)wv[j];
-        load_bwd(K - 2, wv);
-        cp_async_wait_n(D);
-        __syncthreads();
-        const int row = K * 32 + lane;
-        const bool valid = row < n;
-        const int64_t grow = S.row0 + row;
-        for (int d = 1; d <= c; ++d) {
-            const int src = K + d;
-            if (src >= nb) break;
-            const TF* Bs = bufs + (int64_t)(src % nbuf) * brs_max;
-            const TF* T = (d < c) ? Bs + (c - d) * 1024 : Bs;
-            const TF* xs = ring + (int64_t)(src % (c + 1)) * 32 * ld + rhs0;
-#pragma unroll 8
-            for (int r = 0; r < 32; ++r) {
-                A coef = (A)T[tile_idx(r, lane)];
-                if (d == c && r > lane) coef = A(0);
-#pragma unroll
-                for (int j = 0; j < NR; ++j) w[j] -= coef * (A)xs[r * ld + j];
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < NR; ++j) tmp[lane * ld + rhs0 + j] = (TF)w[j];
-        __syncwarp();
-        const TF* B = bufs + (int64_t)(K % nbuf) * brs_max;
-        const A piv = (A)B[c * 1024 + lane];
-        A x[NR];
-#pragma unroll
-        for (int j = 0; j < NR; ++j) x[j] = piv * w[j];
-#pragma unroll 8
-        for (int r = 0; r < 32; ++r) {
-            const A coef = r > lane ? (A)B[tile_idx(r, lane)] : A(0);
-#pragma unroll
-            for (int j = 0; j < NR; ++j) x[j] += coef * (A)tmp[r * ld + rhs0 + j];
-        }
-        TF* xr = ring + (int64_t)(K % (c + 1)) * 32 * ld + rhs0;
-#pragma unroll
-        for (int j = 0; j < NR; ++j) xr[lane * ld + j] = (TF)x[j];
-        if (valid) {
-#pragma unroll
-            for (int j = 0; j < NR; ++j) zf[grow * ld + rhs0 + j] = (TF)x[j];
-        }
-        __syncthreads();
-    };
-#pragma unroll 1
-    for (int K = nb - 1; K >= 0; K -= 2) {
-        bwd_step(K, wb[0]);
-        if (K - 1 >= 0) bwd_step(K - 1, wb[1]);
-    }
 }
 
 // ===========================================================================
@@ -802,65 +545,6 @@ static void norms_ld(const LaunchCtx& L, const double* r, int nrhs) {
 }
 void launch_init_norms(const LaunchCtx& L, const double* r, int nrhs) {
     AMS_DISPATCH_LD(L.ld, norms_ld, L, r, nrhs);
-}
-
-size_t local_solve_smem(int cmax, int ld, size_t tf_bytes, int depth) {
-    return ((size_t)(cmax + depth + 1) * blockrow_elems(cmax) + (size_t)(cmax + 1) * 32 * ld + 32 * ld) *
-           tf_bytes;
-}
-
-// Deepest prefetch (<= 6 block rows) whose staging fits a shared-memory
-// budget that still leaves room for several resident blocks per SM.
-int local_solve_depth(int cmax, int ld, size_t tf_bytes) {
-    const size_t budget = 100 * 1024, hard = 200 * 1024;
-    int d = 4;
-    while (d > 1 && local_solve_smem(cmax, ld, tf_bytes, d) > budget) --d;
-    while (d > 1 && local_solve_smem(cmax, ld, tf_bytes, d) > hard) --d;
-    return d;
-}
-
-template <typename TF, typename TP, int NR, int MM>
-static cudaError_t local_nr(const LocalSolveArgs& a, const void* fac, const void* psi, void* zf,
-                            void* rc) {
-    const int warps = a.ld / NR;
-    const int depth = a.depth > 0 ? a.depth : local_solve_depth(a.cmax, a.ld, sizeof(TF));
-    const size_t smem = local_solve_smem(a.cmax, a.ld, sizeof(TF), depth);
-    auto kern = k_local_solve<TF, TP, NR, MM>;
-    static size_t smem_set = 0;           // per template instance
-    if (smem > smem_set) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        smem_set = smem;
-    }
-    return launch_kernel(a.pdl, kern, dim3(a.nsub), dim3(warps * 32), smem, a.stream, a.subs, (const TF*)fac, a.in.r,
-                         a.in.q, a.in.sc, a.rowscale, (TF*)zf, (const TP*)psi, (TF*)rc, a.ld, a.cmax, depth, a.st);
-}
-
-template <typename TF, typename TP>
-static cudaError_t local_tp(const LocalSolveArgs& a, const void* fac, const void* psi, void* zf, void* rc) {
-    const bool big = a.mmax > 8;
-    const int nrmax = sizeof(TF) == 8 ? (big ? 2 : 4) : (big ? 4 : 8);
-    const int nr = a.ld < nrmax ? a.ld : nrmax;
-    if (big) {
-        switch (nr) {
-            case 1: return local_nr<TF, TP, 1, 16>(a, fac, psi, zf, rc);
-            case 2: return local_nr<TF, TP, 2, 16>(a, fac, psi, zf, rc);
-            default: return local_nr<TF, TP, 4, 16>(a, fac, psi, zf, rc);
-        }
-    }
-    switch (nr) {
-        case 1: return local_nr<TF, TP, 1, 8>(a, fac, psi, zf, rc);
-        case 2: return local_nr<TF, TP, 2, 8>(a, fac, psi, zf, rc);
-        case 4: return local_nr<TF, TP, 4, 8>(a, fac, psi, zf, rc);
-        default: return local_nr<TF, TP, 8, 8>(a, fac, psi, zf, rc);
-    }
-}
-
-cudaError_t launch_local_solve(const LocalSolveArgs& a, int prec, const void* fac, const void* psi,
-                               void* zf, void* rc) {
-    if (prec == AMS_PREC_FP64) return local_tp<double, double>(a, fac, psi, zf, rc);
-    if (prec == AMS_PREC_FP32) return local_tp<float, float>(a, fac, psi, zf, rc);
-    return local_tp<float, __nv_bfloat16>(a, fac, psi, zf, rc);
 }
 
 template <typename TF, typename TP, int LD>

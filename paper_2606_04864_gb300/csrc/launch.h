@@ -69,7 +69,8 @@ struct LocalSolveArgs {
     int mmax;
     const SolveState* st;
     bool pdl;
-    int depth;               // ring depth (block rows in flight); 0: chosen from the band width
+    int depth;               // ring depth (block rows in flight); 0: default
+    int ncols;               // right-hand sides (<= ld); the columns beyond are left as they are
 };
 
 struct LocalTmaArgs {
@@ -130,9 +131,8 @@ void launch_dir_update(const LaunchCtx& L, int prec, const void* z, const double
 void launch_x_flush(const LaunchCtx& L, const double* p, const double* p2, double* x);
 void launch_init_norms(const LaunchCtx& L, const double* r, int nrhs);
 size_t local_solve_smem(int cmax, int ld, size_t tf_bytes, int depth);
-int local_solve_depth(int cmax, int ld, size_t tf_bytes);
-cudaError_t launch_local_solve(const LocalSolveArgs& a, int prec, const void* fac, const void* psi,
-                               void* zf, void* rc);
+// FP64 local solves (k_local_f64.cu)
+cudaError_t launch_local_solve(const LocalSolveArgs& a, const double* fac, const double* psi, double* zf, double* rc);
 void launch_coarse_gemm(const CoarseLaunch& c, int prec, int ld, const void* in, void* out);
 // psif: the basis in fragment order (launch_pack_psi), read by the MMA kernel
 cudaError_t launch_local_tma(const LocalTmaArgs& a, int prec, const void* psi, const void* psif, void* zf, void* rc);
