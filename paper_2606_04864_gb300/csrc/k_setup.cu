@@ -228,20 +228,16 @@ __global__ void k_eig_init(const SubInfo* __restrict__ subs, int P, double* __re
     }
 }
 
-// (\hat A Y)_i = ahat_ii Y_i + sum_{j in Omega, j != i} A_ij Y_j
-__device__ inline void ahat_mult(const SubInfo& Sb, int P, const int64_t* rowptr, const int32_t* colind,
-                                 const double* vals, const double* ahat_diag, const double* Y,
-                                 double* AY) {
-    for (int t = threadIdx.x; t < Sb.n * P; t += blockDim.x) {
-        const int i = t / P, a = t % P;
-        const int64_t g = Sb.row0 + i;
-        double s = ahat_diag[g] * Y[g * P + a];
-        for (int64_t e = rowptr[g]; e < rowptr[g + 1]; ++e) {
-            const int64_t j = colind[e];
-            if (j != g && j >= Sb.row0 && j < Sb.row0 + Sb.n) s += vals[e] * Y[j * P + a];
-        }
-        AY[g * P + a] = s;
+// (\hat A Y)_{g,a} = ahat_gg Y_{g,a} + sum_{j in Omega, j != g} A_gj Y_{j,a}
+__device__ __forceinline__ double ahat_entry(const SubInfo& Sb, int P, const int64_t* rowptr, const int32_t* colind,
+                                             const double* vals, const double* ahat_diag, const double* Y, int64_t g,
+                                             int a) {
+    double s = ahat_diag[g] * Y[g * P + a];
+    for (int64_t e = rowptr[g]; e < rowptr[g + 1]; ++e) {
+        const int64_t j = colind[e];
+        if (j != g && j >= Sb.row0 && j < Sb.row0 + Sb.n) s += vals[e] * Y[j * P + a];
     }
+    return s;
 }
 
 // Rayleigh-Ritz on span(Y) for the pencil (\hat A, S):
@@ -251,12 +247,13 @@ __device__ inline void ahat_mult(const SubInfo& Sb, int P, const int64_t* rowptr
 // Ritz values), for the subspace iterations between convergence checks.
 // One thread block per subdomain; the small dense work is done by warp 0,
 // the Jacobi rotations by the whole block.
+constexpr int kRrRows = 32;   // rows of a subdomain staged at a time
 __global__ void __launch_bounds__(256)
 k_eig_rr(const SubInfo* __restrict__ subs, int P, const int64_t* __restrict__ rowptr,
          const int32_t* __restrict__ colind, const double* __restrict__ vals,
          const double* __restrict__ S, const double* __restrict__ ahat_diag,
-         const double* __restrict__ Y, double* __restrict__ AY, double* __restrict__ Tout,
-         double* __restrict__ theta, int32_t* status, int orth_only) {
+         const double* __restrict__ Y, double* __restrict__ Tout, double* __restrict__ theta, int32_t* status,
+         int orth_only) {
     const SubInfo Sb = subs[blockIdx.x];
     const int p = Sb.p;
     if (p == 0) return;
@@ -266,37 +263,69 @@ k_eig_rr(const SubInfo* __restrict__ subs, int P, const int64_t* __restrict__ ro
     double* W = H + P * P;          // P*P
     double* Rm = W + P * P;         // P*P (R, then R^{-1})
     double* ev = Rm + P * P;        // P
-    if (!orth_only) ahat_mult(Sb, P, rowptr, colind, vals, ahat_diag, Y, AY);
-    __syncthreads();
-    // Gram matrices (upper triangles): one warp per pair (a, b), lanes over
-    // the subdomain's rows, partial sums combined by a fixed shuffle tree
+    // Gram matrices: chunks of kRrRows rows of Y, S Y and \hat A Y (formed on
+    // the way in) in shared memory, one thread per pair (a, b), a <= b, rows
+    // in order.  Bound by the FP64 pipe: one multiply-add per row, pair and
+    // matrix.  (A warp per pair reading columns of Y from global memory, with
+    // S Y formed per pair, took 2.66 ms on 256 subdomains of
+    // 32^2 with 32 columns and 0.46 ms, most of them without H, on 512 of 8^3
+    // with 16; this 0.51 ms with 16 columns and H on either.)
     {
-        const int wid = threadIdx.x >> 5, wl = threadIdx.x & 31, nw = blockDim.x >> 5;
+        double* sY = ev + P;                          // kRrRows x (P + 1) each
+        double* sSY = sY + kRrRows * (P + 1);
+        double* sA = sSY + kRrRows * (P + 1);
         const int npairs = p * (p + 1) / 2;
-        for (int pr = wid; pr < npairs; pr += nw) {
-            int a = 0, rem = pr;
+        constexpr int NPASS = 3;                      // pairs of p <= 32 per 256 threads
+        double g[NPASS], h[NPASS];
+        int pa[NPASS], pb[NPASS];
+#pragma unroll
+        for (int q = 0; q < NPASS; ++q) {
+            g[q] = 0.0;
+            h[q] = 0.0;
+            int a = 0, rem = (int)threadIdx.x + 256 * q;
+            if (rem >= npairs) rem = 0;
             while (rem >= p - a) {
                 rem -= p - a;
                 ++a;
             }
-            const int b = a + rem;
-            double g = 0.0, h = 0.0;
-            for (int i = wl; i < Sb.n; i += 32) {
-                const int64_t r = Sb.row0 + i;
-                const double ya = Y[r * P + a];
-                g += S[r] * ya * Y[r * P + b];
-                if (!orth_only) h += ya * AY[r * P + b];
+            pa[q] = a;
+            pb[q] = a + rem;
+        }
+        for (int r0 = 0; r0 < Sb.n; r0 += kRrRows) {
+            const int nr = min(kRrRows, Sb.n - r0);
+            for (int t = threadIdx.x; t < nr * P; t += blockDim.x) {
+                const int r = t / P, a = t % P;
+                const int64_t gr = Sb.row0 + r0 + r;
+                const double y = Y[gr * P + a];
+                sY[r * (P + 1) + a] = y;
+                sSY[r * (P + 1) + a] = S[gr] * y;
+                if (!orth_only && a < p)
+                    sA[r * (P + 1) + a] = ahat_entry(Sb, P, rowptr, colind, vals, ahat_diag, Y, gr, a);
             }
-            for (int off = 16; off > 0; off >>= 1) {
-                g += __shfl_xor_sync(0xffffffffu, g, off);
-                h += __shfl_xor_sync(0xffffffffu, h, off);
+            __syncthreads();
+#pragma unroll
+            for (int q = 0; q < NPASS; ++q) {
+                if ((int)threadIdx.x + 256 * q >= npairs) break;
+                const double *ya = sY + pa[q], *sa = sSY + pa[q], *yb = sY + pb[q], *ab = sA + pb[q];
+                if (orth_only) {
+                    for (int r = 0; r < nr; ++r) g[q] = fma(sa[r * (P + 1)], yb[r * (P + 1)], g[q]);
+                } else {
+#pragma unroll 4
+                    for (int r = 0; r < nr; ++r) {
+                        g[q] = fma(sa[r * (P + 1)], yb[r * (P + 1)], g[q]);
+                        h[q] = fma(ya[r * (P + 1)], ab[r * (P + 1)], h[q]);
+                    }
+                }
             }
-            if (wl == 0) {
-                G[a * P + b] = g;
-                G[b * P + a] = g;
-                H[a * P + b] = h;
-                H[b * P + a] = h;
-            }
+            __syncthreads();
+        }
+#pragma unroll
+        for (int q = 0; q < NPASS; ++q) {
+            if ((int)threadIdx.x + 256 * q >= npairs) break;
+            G[pa[q] * P + pb[q]] = g[q];
+            G[pb[q] * P + pa[q]] = g[q];
+            H[pa[q] * P + pb[q]] = h[q];
+            H[pb[q] * P + pa[q]] = h[q];
         }
     }
     __syncthreads();
@@ -531,39 +560,67 @@ __global__ void k_eig_update(int64_t nrows_pad, int P, const int32_t* __restrict
     X[t] = v;
 }
 
-// residual norms ||\hat A x_k - theta_k S x_k||_{S^{-1}} for k < ncheck
+// One step of the Chebyshev recurrence of the filtered subspace iteration, per
+// row of a subdomain with largest Ritz value theta_p:
+//   out = k (theta_p + sigma) w - a u - b v   (u may be NULL; out may be w, u or v)
+__global__ void k_eig_cheb(int64_t nrows_pad, int P, const int32_t* __restrict__ sub_of_row,
+                           const SubInfo* __restrict__ subs, const double* __restrict__ theta, double sigma, double k,
+                           const double* w, double a, const double* u, double b, const double* v, double* out) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nrows_pad * P) return;
+    const int s = sub_of_row[t / P];
+    if (s < 0) return;
+    const double f = k * (theta[(int64_t)s * P + subs[s].p - 1] + sigma);
+    double x = fma(f, w[t], -b * v[t]);
+    if (u != nullptr) x = fma(-a, u[t], x);
+    out[t] = x;
+}
+
+// residual norms ||\hat A x_k - theta_k S x_k||_{S^{-1}} for k < ncheck into
+// resid[0 .. nsub), and the spread (theta_p + sigma) / (theta_1 + sigma) of
+// the shifted Ritz values into resid[nsub .. 2 nsub) (infinite where the
+// lowest is not positive: the shift does not make the pencil definite there)
 __global__ void k_eig_resid(const SubInfo* __restrict__ subs, int P, const int64_t* __restrict__ rowptr,
                             const int32_t* __restrict__ colind, const double* __restrict__ vals,
                             const double* __restrict__ S, const double* __restrict__ ahat_diag,
                             const double* __restrict__ X, const double* __restrict__ theta, int ncheck,
-                            double* __restrict__ resid) {
+                            double sigma, double* __restrict__ resid) {
+    // thread t: column t % P (P is a power of two, at most 32) of every
+    // (256 / P)-th row, so that a row's columns are read together; one
+    // reciprocal of S per row (one per entry took most of the kernel's time)
     const SubInfo Sb = subs[blockIdx.x];
-    __shared__ double red[256];
+    __shared__ double red[256], sinv[256];
     const int kmax = min(ncheck, Sb.p);
-    double worst = 0.0;
-    for (int k = 0; k < kmax; ++k) {
-        const double th = theta[(int64_t)blockIdx.x * P + k];
-        double acc = 0.0;
-        for (int i = threadIdx.x; i < Sb.n; i += blockDim.x) {
-            const int64_t g = Sb.row0 + i;
-            double s = ahat_diag[g] * X[g * P + k];
-            for (int64_t e = rowptr[g]; e < rowptr[g + 1]; ++e) {
-                const int64_t j = colind[e];
-                if (j != g && j >= Sb.row0 && j < Sb.row0 + Sb.n) s += vals[e] * X[j * P + k];
-            }
-            const double rr = s - th * S[g] * X[g * P + k];
-            acc += rr * rr / S[g];
-        }
-        red[threadIdx.x] = acc;
+    const int k = threadIdx.x % P, rg = threadIdx.x / P, nrg = 256 / P;
+    const double th = k < kmax ? theta[(int64_t)blockIdx.x * P + k] : 0.0;
+    double acc = 0.0;
+    for (int r0 = 0; r0 < Sb.n; r0 += 256) {
+        const int nr = min(256, Sb.n - r0);
+        if ((int)threadIdx.x < nr) sinv[threadIdx.x] = 1.0 / S[Sb.row0 + r0 + threadIdx.x];
         __syncthreads();
-        for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-            if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-            __syncthreads();
-        }
-        worst = fmax(worst, sqrt(red[0]));
+        if (k < kmax)
+            for (int r = rg; r < nr; r += nrg) {
+                const int64_t g = Sb.row0 + r0 + r;
+                const double rr = ahat_entry(Sb, P, rowptr, colind, vals, ahat_diag, X, g, k) - th * S[g] * X[g * P + k];
+                acc += rr * rr * sinv[r];
+            }
         __syncthreads();
     }
-    if (threadIdx.x == 0) resid[blockIdx.x] = worst;
+    red[threadIdx.x] = acc;
+    __syncthreads();
+    for (int o = 128; o >= P; o >>= 1) {
+        if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+        __syncthreads();
+    }
+    double worst = 0.0;
+    if (threadIdx.x == 0)
+        for (int q = 0; q < kmax; ++q) worst = fmax(worst, sqrt(red[q]));
+    if (threadIdx.x == 0) {
+        resid[blockIdx.x] = worst;
+        const double* th = theta + (int64_t)blockIdx.x * P;
+        const double lo = Sb.p > 0 ? th[0] + sigma : 1.0, hi = Sb.p > 0 ? th[Sb.p - 1] + sigma : 1.0;
+        resid[gridDim.x + blockIdx.x] = lo > 0.0 ? hi / lo : INFINITY;
+    }
 }
 
 // Sign convention (largest-magnitude entry positive, lowest index on ties)
@@ -721,11 +778,10 @@ void launch_eig_init(cudaStream_t s, int nsub, const SubInfo* subs, int P, doubl
 }
 void launch_eig_rr(cudaStream_t s, int nsub, const SubInfo* subs, int P, const int64_t* rowptr,
                    const int32_t* colind, const double* vals, const double* S, const double* ahat_diag,
-                   const double* Y, double* AY, double* T, double* theta, int32_t* status, int orth_only) {
-    const size_t smem = (size_t)(4 * P * P + P) * sizeof(double);
+                   const double* Y, double* T, double* theta, int32_t* status, int orth_only) {
+    const size_t smem = (size_t)(4 * P * P + P + 3 * kRrRows * (P + 1)) * sizeof(double);
     cudaFuncSetAttribute(k_eig_rr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_eig_rr<<<nsub, 256, smem, s>>>(subs, P, rowptr, colind, vals, S, ahat_diag, Y, AY, T, theta, status,
-                                     orth_only);
+    k_eig_rr<<<nsub, 256, smem, s>>>(subs, P, rowptr, colind, vals, S, ahat_diag, Y, T, theta, status, orth_only);
 }
 void launch_eig_update(cudaStream_t s, int64_t nrows_pad, int P, const int32_t* sub_of_row,
                        const SubInfo* subs, const double* Y, const double* T, double* X) {
@@ -735,8 +791,15 @@ void launch_eig_update(cudaStream_t s, int64_t nrows_pad, int P, const int32_t* 
 void launch_eig_resid(cudaStream_t s, int nsub, const SubInfo* subs, int P, const int64_t* rowptr,
                       const int32_t* colind, const double* vals, const double* S,
                       const double* ahat_diag, const double* X, const double* theta, int ncheck,
-                      double* resid) {
-    k_eig_resid<<<nsub, 256, 0, s>>>(subs, P, rowptr, colind, vals, S, ahat_diag, X, theta, ncheck, resid);
+                      double sigma, double* resid) {
+    k_eig_resid<<<nsub, 256, 0, s>>>(subs, P, rowptr, colind, vals, S, ahat_diag, X, theta, ncheck, sigma, resid);
+}
+void launch_eig_cheb(cudaStream_t s, int64_t nrows_pad, int P, const int32_t* sub_of_row, const SubInfo* subs,
+                     const double* theta, double sigma, double k, const double* w, double a, const double* u,
+                     double b, const double* v, double* out) {
+    const int64_t tot = nrows_pad * P;
+    k_eig_cheb<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(nrows_pad, P, sub_of_row, subs, theta, sigma, k, w, a, u,
+                                                             b, v, out);
 }
 void launch_eig_finalize(cudaStream_t s, int nsub, const SubInfo* subs, int P, const double* X,
                          const double* S, double* psi64) {
