@@ -71,15 +71,6 @@ namespace ams {
 // banks in each quarter warp.
 __device__ __forceinline__ int bswz(int rho) { return ((rho & 1) ? 5 : 0) ^ (rho & 2); }
 
-// x = head + tail, head TF32 (nearest, ties away); the tail is exact in FP32
-// with at most 12 significant bits and goes to the MMA as it is: the unit
-// drops its last bit, the same error as rounding it to TF32 first.  A NaN or
-// infinity comes back as a NaN tail.
-__device__ __forceinline__ void split_fast(float x, uint32_t& hi, uint32_t& lo) {
-    hi = (__float_as_uint(x) + 0x1000u) & 0xffffe000u;
-    lo = __float_as_uint(x - __uint_as_float(hi));
-}
-
 // Which fragments (16 rows x 8 columns of the operand) a triangular mask
 // empties.  MODE 0 all, 1 keep q >= r (L_{K,K-c}), 2 keep q < r (strict lower
 // part, L_KK^{-1}); TR: the operand is the transposed tile.
@@ -146,7 +137,7 @@ __device__ __forceinline__ void half_mma(const float* T, const uint4* B, const L
         }
         uint32_t ah[4], al[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) split_fast(a[i], ah[i], al[i]);
+        for (int i = 0; i < 4; ++i) split_tf32(a[i], ah[i], al[i]);
 #pragma unroll
         for (int nf = 0; nf < NF; ++nf) mma_tf32(acc[nf], al, b[nf].x, b[nf].y);
 #pragma unroll
@@ -186,8 +177,8 @@ __device__ __forceinline__ void put_block(uint4* B, int wr, const float (&v)[NF]
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
             uint4 u;
-            split_fast(v[nf][j], u.x, u.z);
-            split_fast(v[nf][2 + j], u.y, u.w);
+            split_tf32(v[nf][j], u.x, u.z);
+            split_tf32(v[nf][2 + j], u.y, u.w);
             B[(wr ^ j) + 8 * nf] = u;
         }
 }
@@ -402,7 +393,7 @@ k_local_mma(const float* __restrict__ tiles_g, const SubInfo* __restrict__ subs,
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     if (sizeof(TP) == 2) ah[i] = __float_as_uint(a[i]);   // BF16 entries are exact in TF32
-                    else split_fast(a[i], ah[i], alo[i]);
+                    else split_tf32(a[i], ah[i], alo[i]);
                 }
 #pragma unroll
                 for (int nf = 0; nf < NF; ++nf) {

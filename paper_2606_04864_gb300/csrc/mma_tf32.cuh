@@ -8,16 +8,16 @@
 
 namespace ams {
 
-// TF32 value (as its 32-bit pattern) nearest to x
-__device__ __forceinline__ uint32_t to_tf32(float x) {
-    uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;\n" : "=r"(r) : "f"(x));
-    return r;
-}
-// x = head + tail (+ below FP32 resolution), head and tail TF32
+// x = head + tail, the head TF32 (nearest, ties away).  The tail is exact in
+// FP32 with at most 12 significant bits and goes to the MMA as it is: the
+// unit drops its last bit, the same error as rounding it to TF32 first.  Three
+// operations at the ALU's rate; two cvt.rna instructions, at a quarter of it,
+// made the kernels that split on the fly issue-bound (coarse products at 32
+// right-hand sides, N_c = 24,576: 322 -> 279 us).  A NaN or
+// infinity comes back as a NaN tail.
 __device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo) {
-    hi = to_tf32(x);
-    lo = to_tf32(x - __uint_as_float(hi));
+    hi = (__float_as_uint(x) + 0x1000u) & 0xffffe000u;
+    lo = __float_as_uint(x - __uint_as_float(hi));
 }
 // d += a b, a 16x8 (row), b 8x8 (col), TF32 in, FP32 accumulate
 __device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
