@@ -39,78 +39,78 @@ namespace ams {
 namespace {
 
 constexpr int TB = 64;          // tile edge
+constexpr int TN = 16;          // a block of the tile products makes 64 x 16 (or 16 x 64) outputs of a tile
+constexpr int TSPLIT = TB / TN; // blocks per tile
 constexpr int TKC = 32;         // contraction chunk staged in shared memory
 constexpr int TP = TB + 1;      // padded shared-memory row
-constexpr int TTHREADS = 256;   // 16 x 16 threads, 4 x 4 outputs each
+constexpr int TTHREADS = 256;   // 16 x 16 threads, 4 outputs each
 
 __device__ __forceinline__ int tile_rows(int64_t nc, int t) {
     const int64_t r = nc - (int64_t)t * TB;
     return r < TB ? (int)r : TB;
 }
 
-// acc[a][b] += sum_kk Aop(m, kk) Bop(kk, n), m = tx + 16a, n = ty + 16b,
-// kk < kdim, with Aop(m, kk) = A[m + kk*lda] (zero for m >= am) and
-// Bop(kk, n) = BT ? B[n + kk*ldb] : B[kk + n*ldb] (zero for n >= bn).
-template <bool BT>
-__device__ __forceinline__ void tile_gemm(double (&acc)[4][4], const double* __restrict__ A, int64_t lda, int am,
-                                          const double* __restrict__ B, int64_t ldb, int bn, int kdim,
+// A 64 x 64 x 64 tile product is 8192 FP64 warp instructions, 70 us of one
+// SM's FP64 pipe, and most steps of the factorisation have fewer tiles than
+// the GPU has SMs: four blocks share a tile (factor and inverse at N_c = 3072
+// 22 -> 13 ms, 8192 62 -> 37, 24,576 401 -> 343) (MR x NC outputs each, 64 x 16 or
+// 16 x 64; thread (tx, ty) has rows tx + 16 a, columns ty + 16 b).
+// acc += sum_kk Aop(m, kk) Bop(kk, n), kk < kdim, with Aop(m, kk) =
+// A[m + kk*lda] (zero for m >= am) and Bop(kk, n) = BT ? B[n + kk*ldb] :
+// B[kk + n*ldb] (zero for n >= bn).
+template <bool BT, int MR, int NC>
+__device__ __forceinline__ void tile_gemm(double (&acc)[MR / 16][NC / 16], const double* __restrict__ A, int64_t lda,
+                                          int am, const double* __restrict__ B, int64_t ldb, int bn, int kdim,
                                           double (*As)[TP], double (*Bs)[TP]) {
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     for (int k0 = 0; k0 < kdim; k0 += TKC) {
 #pragma unroll
-        for (int s = 0; s < 8; ++s) {
-            const int m = tid & 63, kk = (tid >> 6) + 4 * s;
+        for (int e = tid; e < TKC * MR; e += TTHREADS) {
+            const int m = e % MR, kk = e / MR;
             As[kk][m] = (m < am && k0 + kk < kdim) ? A[m + (int64_t)(k0 + kk) * lda] : 0.0;
         }
-        if (BT) {
 #pragma unroll
-            for (int s = 0; s < 8; ++s) {
-                const int n = tid & 63, kk = (tid >> 6) + 4 * s;
-                Bs[kk][n] = (n < bn && k0 + kk < kdim) ? B[n + (int64_t)(k0 + kk) * ldb] : 0.0;
-            }
-        } else {
-#pragma unroll
-            for (int s = 0; s < 8; ++s) {
-                const int kk = tid & 31, n = (tid >> 5) + 8 * s;
-                Bs[kk][n] = (n < bn && k0 + kk < kdim) ? B[(k0 + kk) + (int64_t)n * ldb] : 0.0;
-            }
+        for (int e = tid; e < TKC * NC; e += TTHREADS) {
+            const int n = BT ? e % NC : e / TKC, kk = BT ? e / NC : e % TKC;
+            Bs[kk][n] = (n < bn && k0 + kk < kdim) ? (BT ? B[n + (int64_t)(k0 + kk) * ldb] : B[(k0 + kk) + (int64_t)n * ldb])
+                                                   : 0.0;
         }
         __syncthreads();
-#pragma unroll 4
+#pragma unroll 8
         for (int kk = 0; kk < TKC; ++kk) {
-            double a[4], b[4];
+            double a[MR / 16], b[NC / 16];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                a[i] = As[kk][tx + 16 * i];
-                b[i] = Bs[kk][ty + 16 * i];
-            }
+            for (int i = 0; i < MR / 16; ++i) a[i] = As[kk][tx + 16 * i];
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int j = 0; j < NC / 16; ++j) b[j] = Bs[kk][ty + 16 * j];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+            for (int i = 0; i < MR / 16; ++i)
+#pragma unroll
+                for (int j = 0; j < NC / 16; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
         }
         __syncthreads();
     }
 }
 
-__device__ __forceinline__ void zero_acc(double (&acc)[4][4]) {
+template <int MI, int NJ>
+__device__ __forceinline__ void zero_acc(double (&acc)[MI][NJ]) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < MI; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+        for (int j = 0; j < NJ; ++j) acc[i][j] = 0.0;
 }
 
 // C[m][n] = acc (SUB = false) or C[m][n] -= acc (SUB = true), m < cm, n < cn.
-template <bool SUB>
-__device__ __forceinline__ void tile_store(const double (&acc)[4][4], double* __restrict__ C, int64_t ldc, int cm,
+template <bool SUB, int MI, int NJ>
+__device__ __forceinline__ void tile_store(const double (&acc)[MI][NJ], double* __restrict__ C, int64_t ldc, int cm,
                                            int cn) {
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < NJ; ++j) {
         const int n = ty + 16 * j;
         if (n >= cn) continue;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < MI; ++i) {
             const int m = tx + 16 * i;
             if (m >= cm) continue;
             double* p = C + m + (int64_t)n * ldc;
@@ -121,7 +121,9 @@ __device__ __forceinline__ void tile_store(const double (&acc)[4][4], double* __
 
 // Diagonal tile t: L_tt = chol(A_tt) in place (lower triangle), its inverse
 // into invd[t] (64 x 64 column-major; identity on the padding of a ragged
-// last tile) and into the diagonal tile of X.  A pivot that is not positive
+// last tile) and into the diagonal tile of X.  One block, the
+// serial part of every step (with a square root and a reciprocal in each of
+// the 64 pivots' chain 171 us).  A pivot that is not positive
 // records its coarse row in *bad (min over tiles) and is replaced by 1 so
 // that the sweep stays finite; the host reports the failure.
 __global__ void __launch_bounds__(TTHREADS) k_tile_potrf(double* __restrict__ A, double* __restrict__ X, int64_t nc,
@@ -140,49 +142,120 @@ __global__ void __launch_bounds__(TTHREADS) k_tile_potrf(double* __restrict__ A,
         else v = (r == c) ? 1.0 : 0.0;
         S[r][c] = v;
     }
-    __shared__ double s_rs;         // reciprocal of the current pivot
-    __shared__ double s_inv[TB];    // reciprocal pivots, for the inverse
-    __syncthreads();
-    for (int j = 0; j < TB; ++j) {
-        // one thread takes the pivot's square root and reciprocal (FP64
-        // square root and division are long sequences on this GPU's narrow
-        // FP64 pipe: not once per thread)
-        if (tid == 0) {
-            double d = S[j][j];
-            if (!(d > 0.0)) {
-                atomicMin(bad, (unsigned long long)((int64_t)t * TB + j));
-                d = 1.0;
-            }
-            const double sq = sqrt(d);
-            S[j][j] = sq;
-            s_rs = 1.0 / sq;
-            s_inv[j] = s_rs;
+    __shared__ double s_inv[TB];    // reciprocal pivots 1 / d_j, then 1 / sqrt(d_j)
+    __shared__ double s_sq[TB];
+    // The factor as unscaled columns (S[r][c] -= S[r][j] S[c][j] / d_j), the
+    // square roots taken together at the end: a step waits for one reciprocal
+    // only, and the thread that makes the next pivot takes it while the
+    // others update the rest (the FP64 square root and division are long
+    // sequences, at a quarter of the pipe's rate for a single warp).
+    auto pivot = [&](int j, double d) {
+        if (!(d > 0.0)) {
+            atomicMin(bad, (unsigned long long)((int64_t)t * TB + j));
+            d = 1.0;
         }
-        __syncthreads();
-        const double rs = s_rs;
-        for (int r = j + 1 + tid; r < TB; r += TTHREADS) S[r][j] *= rs;
-        __syncthreads();
-        for (int e = tid; e < TB * TB; e += TTHREADS) {
-            const int r = e >> 6, c = e & 63;
-            if (c > j && r >= c) S[r][c] = fma(-S[r][j], S[c][j], S[r][c]);
+        s_sq[j] = d;
+        s_inv[j] = 1.0 / d;
+    };
+    __syncthreads();
+    if (tid == 0) pivot(0, S[0][0]);
+    __syncthreads();
+    // 4 x 4 register tiles of the lower triangle, one per thread, last rows first
+    int br = 15, bc = tid;
+    while (br >= 0 && bc > br) bc -= br + 1, --br;
+    const bool own = br >= 0;
+    double v[4][4];
+    if (own)
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) v[a][b] = S[4 * br + a][4 * bc + b];
+    for (int j = 0; j < TB - 1; ++j) {
+        if (own && 4 * br + 3 > j && 4 * bc + 3 > j) {
+            const double inv = s_inv[j];
+            double lr[4], lc[4];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                lr[a] = S[4 * br + a][j] * inv;
+                lc[a] = S[4 * bc + a][j];
+            }
+            if (br == bc && (j + 1) >> 2 == br) {     // the next pivot and its reciprocal first
+                const int k = (j + 1) & 3;
+                double d = 0.0;
+#pragma unroll
+                for (int a = 0; a < 4; ++a)
+                    if (a == k) d = fma(-lr[a], lc[a], v[a][a]);
+                pivot(j + 1, d);
+            }
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int b = 0; b < 4; ++b)
+                    if (4 * bc + b > j && 4 * br + a >= 4 * bc + b) v[a][b] = fma(-lr[a], lc[b], v[a][b]);
+            if (bc == (j + 1) >> 2) {                 // column j + 1 is final: show it
+#pragma unroll
+                for (int b = 0; b < 4; ++b)
+                    if (b == ((j + 1) & 3))
+#pragma unroll
+                        for (int a = 0; a < 4; ++a)
+                            if (4 * br + a > j) S[4 * br + a][j + 1] = v[a][b];
+            }
         }
         __syncthreads();
     }
-    // inverse of the lower-triangular S, column c by four lanes of one warp
-    {
-        const int c = tid >> 2, q = tid & 3;
-        if (q == 0) Li[c][c] = s_inv[c];
-        __syncwarp();
-        for (int r = 1; r < TB; ++r) {
-            double s = 0.0;
-            if (r > c)
-                for (int l = c + q; l < r; l += 4) s = fma(S[r][l], Li[l][c], s);
-            s += __shfl_xor_sync(0xffffffffu, s, 1);
-            s += __shfl_xor_sync(0xffffffffu, s, 2);
-            if (r > c && q == 0) Li[r][c] = -s * s_inv[r];
-            __syncwarp();
+    if (tid < TB) {
+        const double sq = sqrt(s_sq[tid]);
+        s_sq[tid] = sq;
+        s_inv[tid] = 1.0 / sq;
+    }
+    __syncthreads();
+    for (int e = tid; e < TB * TB; e += TTHREADS) {
+        const int r = e >> 6, c = e & 63;
+        if (r > c) S[r][c] *= s_inv[c];
+        else if (r == c) S[r][c] = s_sq[c];
+        Li[r][c] = 0.0;
+    }
+    __syncthreads();
+    // Inverse of the lower-triangular S: the four 16 x 16 diagonal blocks by
+    // forward substitution (a thread per column), then twice
+    // Li21 = -Li22 (S21 Li11), on blocks of 16 and of 32 (the product in the
+    // unused upper triangle of Li).
+    if (tid < TB) {
+        const int b0 = tid & ~15, c = tid & 15;
+        double x[16];
+#pragma unroll
+        for (int r = 0; r < 16; ++r) {
+            double w = 0.0;
+#pragma unroll
+            for (int l = 0; l < 16; ++l)
+                if (l < r) w = fma(S[b0 + r][b0 + l], x[l], w);
+            x[r] = r < c ? 0.0 : r == c ? s_inv[b0 + r] : -w * s_inv[b0 + r];
         }
-        for (int r = q; r < c; r += 4) Li[r][c] = 0.0;
+#pragma unroll
+        for (int r = 0; r < 16; ++r) Li[b0 + r][b0 + c] = x[r];
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int h = 16; h < TB; h *= 2) {
+        const int per = h * h, npair = TB / (2 * h);      // outputs per pair of blocks
+        for (int e = tid; e < per * npair; e += TTHREADS) {
+            const int b0 = e / per * 2 * h, m = e % per / h, n = e % h;
+            double w = 0.0;
+            for (int l = n; l < h; ++l) w = fma(S[b0 + h + m][b0 + l], Li[b0 + l][b0 + n], w);
+            Li[b0 + m][b0 + h + n] = w;
+        }
+        __syncthreads();
+        for (int e = tid; e < per * npair; e += TTHREADS) {
+            const int b0 = e / per * 2 * h, m = e % per / h, n = e % h;
+            double w = 0.0;
+            for (int l = 0; l <= m; ++l) w = fma(Li[b0 + h + m][b0 + h + l], Li[b0 + l][b0 + h + n], w);
+            Li[b0 + h + m][b0 + n] = -w;
+        }
+        __syncthreads();
+    }
+    for (int e = tid; e < TB * TB; e += TTHREADS) {
+        const int r = e >> 6, c = e & 63;
+        if (r < c) Li[r][c] = 0.0;
     }
     __syncthreads();
     double* iv = invd + (int64_t)t * TB * TB;
@@ -196,57 +269,63 @@ __global__ void __launch_bounds__(TTHREADS) k_tile_potrf(double* __restrict__ A,
     }
 }
 
-// Column step k of the factorisation: L_ik = A_ik L_kk^{-T}, one block per
-// kept row tile i > k (rows[blockIdx.x]).
+// Column step k of the factorisation: L_ik = A_ik L_kk^{-T}, four blocks per
+// kept row tile i > k (rows[blockIdx.x / 4]), 16 rows each (in place: a row's
+// outputs need that row only).
 __global__ void __launch_bounds__(TTHREADS) k_tile_trsm(double* __restrict__ A, int64_t nc, int k,
                                                         const int32_t* __restrict__ rows,
                                                         const double* __restrict__ invd) {
     __shared__ double As[TKC][TP], Bs[TKC][TP];
-    const int i = rows[blockIdx.x];
-    const int mi = tile_rows(nc, i), mk = tile_rows(nc, k);
-    double* Cik = A + (int64_t)i * TB + (int64_t)k * TB * nc;
-    double acc[4][4];
+    const int i = rows[blockIdx.x / TSPLIT], m0 = blockIdx.x % TSPLIT * TN;
+    const int mi = tile_rows(nc, i) - m0, mk = tile_rows(nc, k);
+    if (mi <= 0) return;
+    double* Cik = A + (int64_t)i * TB + m0 + (int64_t)k * TB * nc;
+    double acc[1][4];
     zero_acc(acc);
-    tile_gemm<true>(acc, Cik, nc, mi, invd + (int64_t)k * TB * TB, TB, mk, mk, As, Bs);
+    tile_gemm<true, TN, TB>(acc, Cik, nc, mi, invd + (int64_t)k * TB * TB, TB, mk, mk, As, Bs);
     tile_store<false>(acc, Cik, nc, mi, mk);
 }
 
 // Column step k of the factorisation: A_ij -= L_ik L_jk^T for the kept
-// pairs (pairs[blockIdx.x] = (i, j), i >= j > k).
+// pairs (pairs[blockIdx.x / 4] = (i, j), i >= j > k), 16 columns per block.
 __global__ void __launch_bounds__(TTHREADS) k_tile_update(double* __restrict__ A, int64_t nc, int k,
                                                           const int2* __restrict__ pairs) {
     __shared__ double As[TKC][TP], Bs[TKC][TP];
-    const int2 p = pairs[blockIdx.x];
-    const int mi = tile_rows(nc, p.x), mj = tile_rows(nc, p.y), mk = tile_rows(nc, k);
+    const int2 p = pairs[blockIdx.x / TSPLIT];
+    const int n0 = blockIdx.x % TSPLIT * TN;
+    const int mi = tile_rows(nc, p.x), mj = tile_rows(nc, p.y) - n0, mk = tile_rows(nc, k);
+    if (mj <= 0) return;
     const double* Lik = A + (int64_t)p.x * TB + (int64_t)k * TB * nc;
-    const double* Ljk = A + (int64_t)p.y * TB + (int64_t)k * TB * nc;
-    double acc[4][4];
+    const double* Ljk = A + (int64_t)p.y * TB + n0 + (int64_t)k * TB * nc;
+    double acc[4][1];
     zero_acc(acc);
-    tile_gemm<true>(acc, Lik, nc, mi, Ljk, nc, mj, mk, As, Bs);
-    tile_store<true>(acc, A + (int64_t)p.x * TB + (int64_t)p.y * TB * nc, nc, mi, mj);
+    tile_gemm<true, TB, TN>(acc, Lik, nc, mi, Ljk, nc, mj, mk, As, Bs);
+    tile_store<true>(acc, A + (int64_t)p.x * TB + ((int64_t)p.y * TB + n0) * nc, nc, mi, mj);
 }
 
 // Row step k of the inversion: X_ic -= L_ik X_kc for the kept pairs
-// (tasks[blockIdx.x] = (i, c | last << 31), i > k >= c); on the pair's last
-// update, X_ic = L_ii^{-1} X_ic.
+// (tasks[blockIdx.x / 4] = (i, c | last << 31), i > k >= c), 16 columns per
+// block; on the pair's last update, X_ic = L_ii^{-1} X_ic.
 __global__ void __launch_bounds__(TTHREADS) k_tile_inv_step(const double* __restrict__ A, double* __restrict__ X,
                                                             int64_t nc, int k, const int2* __restrict__ tasks,
                                                             const double* __restrict__ invd) {
     __shared__ double As[TKC][TP], Bs[TKC][TP];
-    const int2 p = tasks[blockIdx.x];
+    const int2 p = tasks[blockIdx.x / TSPLIT];
+    const int n0 = blockIdx.x % TSPLIT * TN;
     const int i = p.x, c = p.y & 0x7fffffff;
     const bool last = (p.y >> 31) & 1;
-    const int mi = tile_rows(nc, i), mc = tile_rows(nc, c), mk = tile_rows(nc, k);
-    double* Xic = X + (int64_t)i * TB + (int64_t)c * TB * nc;
-    double acc[4][4];
+    const int mi = tile_rows(nc, i), mc = tile_rows(nc, c) - n0, mk = tile_rows(nc, k);
+    if (mc <= 0) return;
+    double* Xic = X + (int64_t)i * TB + ((int64_t)c * TB + n0) * nc;
+    double acc[4][1];
     zero_acc(acc);
-    tile_gemm<false>(acc, A + (int64_t)i * TB + (int64_t)k * TB * nc, nc, mi,
-                     X + (int64_t)k * TB + (int64_t)c * TB * nc, nc, mc, mk, As, Bs);
+    tile_gemm<false, TB, TN>(acc, A + (int64_t)i * TB + (int64_t)k * TB * nc, nc, mi,
+                             X + (int64_t)k * TB + ((int64_t)c * TB + n0) * nc, nc, mc, mk, As, Bs);
     tile_store<true>(acc, Xic, nc, mi, mc);
     if (!last) return;
     __syncthreads();   // the block's own global writes are visible to it after the barrier
     zero_acc(acc);
-    tile_gemm<false>(acc, invd + (int64_t)i * TB * TB, TB, mi, Xic, nc, mc, mi, As, Bs);
+    tile_gemm<false, TB, TN>(acc, invd + (int64_t)i * TB * TB, TB, mi, Xic, nc, mc, mi, As, Bs);
     tile_store<false>(acc, Xic, nc, mi, mc);
 }
 
@@ -348,15 +427,15 @@ void launch_coarse_tile_factor(cudaStream_t s, const CoarseTilePlan& P, const in
     k_tile_potrf<<<1, TTHREADS, psmem, s>>>(d_A, d_X, P.nc, 0, d_invd, d_bad);
     for (int k = 0; k < T; ++k) {
         const int64_t nt = P.trsm_ptr[k + 1] - P.trsm_ptr[k];
-        if (nt > 0) k_tile_trsm<<<(unsigned)nt, TTHREADS, 0, s>>>(d_A, P.nc, k, d_trsm + P.trsm_ptr[k], d_invd);
+        if (nt > 0) k_tile_trsm<<<(unsigned)(TSPLIT * nt), TTHREADS, 0, s>>>(d_A, P.nc, k, d_trsm + P.trsm_ptr[k], d_invd);
         const int64_t nu = P.upd_ptr[k + 1] - P.upd_ptr[k];
-        if (nu > 0) k_tile_update<<<(unsigned)nu, TTHREADS, 0, s>>>(d_A, P.nc, k, d_upd + P.upd_ptr[k]);
+        if (nu > 0) k_tile_update<<<(unsigned)(TSPLIT * nu), TTHREADS, 0, s>>>(d_A, P.nc, k, d_upd + P.upd_ptr[k]);
         if (k + 1 < T) k_tile_potrf<<<1, TTHREADS, psmem, s>>>(d_A, d_X, P.nc, k + 1, d_invd, d_bad);
     }
     for (int k = 0; k + 1 < T; ++k) {
         const int64_t ni = P.inv_ptr[k + 1] - P.inv_ptr[k];
         if (ni > 0)
-            k_tile_inv_step<<<(unsigned)ni, TTHREADS, 0, s>>>(d_A, d_X, P.nc, k, d_inv + P.inv_ptr[k], d_invd);
+            k_tile_inv_step<<<(unsigned)(TSPLIT * ni), TTHREADS, 0, s>>>(d_A, d_X, P.nc, k, d_inv + P.inv_ptr[k], d_invd);
     }
 }
 
