@@ -1791,23 +1791,32 @@ static ams_status autotune(ams_handle h, const double* f_dev, int nrhs, int ld) 
         launch_direction_spmv(h, L, h->d_p, h->d_p2);
         return AMS_OK;
     };
-    {   // local-solve ring depth, among the depths whose staging fits 200 KB
+    {   // local-solve ring depth (staging within 200 KB) and right-hand sides per column group together:
+        // the right depth depends on the group's size.  The right-looking kernels (all but the one-RHS
+        // one) gain nothing from more than a few rows in flight and lose occupancy to them.
         const ResidIn in{h->d_r, h->d_q, h->d_sc};
+        const bool one_rhs = h->use_tma && ld == 1, groups = h->use_tma && ld >= 16;
+        const int dmin = h->use_tma ? 2 : 1, dmax = one_rhs ? 6 : h->use_tma ? 4 : 3;
         float best = 1e30f;
-        int arg = 0;
-        for (int d = 1; d <= 6; ++d) {
-            const size_t smem = h->use_tma ? local_tma_launch_smem(local_tma_args(h, ld, in, true), d)
-                                           : local_solve_smem(h->cmax, ld, h->tf_bytes(), d);
-            if (smem > 200 * 1024 || (h->use_tma && d < 2)) continue;
-            T.depth = d;
-            float ms = 0.f;
-            AMS_TRY(timed_after(spmv, [&]() -> ams_status { return launch_local(h, ld, in, true); }, &ms));
-            if (ms < best) {
-                best = ms;
-                arg = d;
+        int arg = 0, argn = 0;
+        for (int nr = groups ? 16 : 0; nr == 0 || nr >= 8; nr = nr == 0 ? 1 : nr / 2) {
+            for (int d = dmin; d <= dmax; ++d) {
+                const size_t smem = h->use_tma ? local_tma_launch_smem(local_tma_args(h, ld, in, true), d)
+                                               : local_solve_smem(h->cmax, ld, h->tf_bytes(), d);
+                if (smem > 200 * 1024) continue;
+                T.depth = d;
+                T.nr = nr;
+                float ms = 0.f;
+                AMS_TRY(timed_after(spmv, [&]() -> ams_status { return launch_local(h, ld, in, true); }, &ms));
+                if (ms < best) {
+                    best = ms;
+                    arg = d;
+                    argn = nr;
+                }
             }
         }
         T.depth = arg;
+        T.nr = argn;
     }
     if (h->use_tma && ld == 1) {   // one-RHS local solve: L2 priorities of the factor tiles
         const ResidIn in{h->d_r, h->d_q, h->d_sc};
@@ -1826,21 +1835,6 @@ static ams_status autotune(ams_handle h, const double* f_dev, int nrhs, int ld) 
         }
         T.l2mode = cand[arg][0];
         T.l2keep = cand[arg][1];
-    }
-    if (h->use_tma && ld >= 16) {   // several-RHS local solve: right-hand sides per column group
-        const ResidIn in{h->d_r, h->d_q, h->d_sc};
-        float best = 1e30f;
-        int arg = 0;
-        for (int nr = 16; nr >= 8; nr /= 2) {
-            T.nr = nr;
-            float ms = 0.f;
-            AMS_TRY(timed_after(spmv, [&]() -> ams_status { return launch_local(h, ld, in, true); }, &ms));
-            if (ms < best) {
-                best = ms;
-                arg = nr;
-            }
-        }
-        T.nr = arg;
     }
     {   // subdomain layout: prolongation (updates x and r of this throw-away state)
         float best = 1e30f;

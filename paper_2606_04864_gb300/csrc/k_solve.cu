@@ -169,18 +169,31 @@ k_x_flush(const double* __restrict__ p, const double* __restrict__ p2, double* _
 // mode 0: z only (a plain preconditioner application).
 // mode 1: first application of a solve: z and rho = r.z (beta = 0).
 // mode 2: CG iteration.  For (system, rhs) pairs still iterating,
-//         r <- r - alpha q and x <- x + alpha p with alpha = rho / pq (the
-//         local solves applied the same fused multiply-add to r on the fly),
-//         then r.z, r.r and, for flexible CG, z.q; the last block of a
+//         r <- r - alpha q and (up to four right-hand sides) x <- x + alpha p
+//         with alpha = rho / pq (the local solves applied the same fused
+//         multiply-add to r on the fly), then r.z, r.r and, for flexible CG,
+//         z.q; the last block of a
 //         system applies the convergence test and sets beta: rho'/rho (PCG)
 //         or -(z.q)/(p.q) (flexible CG).
 // ===========================================================================
-// Basis row of `m` entries into registers; one 16-byte load per 16 bytes
-// when the row is 16-byte aligned and m == MM.
+// Basis row of `m` entries into registers: one 16-byte load per 16 bytes when
+// the row is 16-byte aligned and m == MM (vec = 2), pairs of entries when m is
+// even and pairs are aligned (vec = 1), else entry by entry.
 template <typename TP, int MM>
-__device__ __forceinline__ void load_basis_row(const TP* __restrict__ pr, int m, bool vec, TP (&v)[MM]) {
+__device__ __forceinline__ void load_basis_row(const TP* __restrict__ pr, int m, int vec, TP (&v)[MM]) {
     constexpr int PER = 16 / sizeof(TP);
-    if (MM % PER == 0 && vec) {
+    using P2 = typename std::conditional<sizeof(TP) == 2, uint32_t,
+                                         typename std::conditional<sizeof(TP) == 4, uint2, uint4>::type>::type;
+    if (vec == 1) {
+#pragma unroll
+        for (int k = 0; k < MM; k += 2) {
+            P2 u{};
+            if (k < m) u = __ldg(reinterpret_cast<const P2*>(pr + k));
+            const TP* t = reinterpret_cast<const TP*>(&u);
+            v[k] = t[0];
+            v[k + 1] = t[1];
+        }
+    } else if (MM % PER == 0 && vec == 2) {
 #pragma unroll
         for (int k = 0; k < MM; k += PER) {
             const uint4 u = __ldg(reinterpret_cast<const uint4*>(pr + k));
@@ -194,13 +207,20 @@ __device__ __forceinline__ void load_basis_row(const TP* __restrict__ pr, int m,
     }
 }
 
-template <typename TF, typename TP, int LD, int MM>
-__global__ void __launch_bounds__(kRedThreads)
+// MODE: 0 and 1 as above, 2 an iteration of PCG, 3 of flexible CG.  Bound by the
+// FP64 pipe (two thirds busy at 16 and more right-hand sides: r', three dots)
+// and the latency of its streams: the four elements a thread has in flight need
+// the loads free of branches (the mode as a run-time argument: 128^3 x 32 785
+// us, 96x80x72 x 3 78; this 735 and 72) and 64 registers, four blocks per SM
+// (two elements and six blocks 803 and 79, one and eight 834 and 79).
+template <typename TF, typename TP, int LD, int MM, int MODE>
+__global__ void __launch_bounds__(kRedThreads, 4)
 k_prolong_update(const SubInfo* __restrict__ subs, const TP* __restrict__ psi, const TF* __restrict__ ec,
                  const TF* __restrict__ yc, const TF* __restrict__ qmat, const CoarseRef* __restrict__ cref, const int32_t* __restrict__ gat,
                  const TF* __restrict__ zf, double* __restrict__ r, const double* __restrict__ q,
                  double* __restrict__ x, const double* __restrict__ p, TF* __restrict__ z, RedLayout R,
-                 CgScalars* sc, SolveState* st, int nseg, int flexible, int mode) {
+                 CgScalars* sc, SolveState* st, int nseg) {
+    constexpr bool ITER = MODE >= 2, FLEX = MODE == 3, XUPD = ITER && LD < 8;
     using AT = typename Acc<TF>::type;
     using V4 = typename std::conditional<sizeof(TF) == 4, float4, double4>::type;
     constexpr int NCG = kRedThreads / LD;            // column groups of the backward product
@@ -217,7 +237,7 @@ k_prolong_update(const SubInfo* __restrict__ subs, const TP* __restrict__ psi, c
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double alpha = 0.0;
     bool upd = false;
-    if (mode == 2) {
+    if (ITER) {
         const CgScalars c = sc[(int64_t)R.blk_seg[blockIdx.x] * LD + rhs];
         upd = c.active != 0;
         if (upd) alpha = c.alpha;
@@ -274,7 +294,8 @@ k_prolong_update(const SubInfo* __restrict__ subs, const TP* __restrict__ psi, c
             }
         }
         __syncthreads();
-        const bool vec = (m == MM) && ((reinterpret_cast<uintptr_t>(psi + S.psi_off) & 15) == 0);
+        const uintptr_t pa = reinterpret_cast<uintptr_t>(psi + S.psi_off);
+        const int vec = m == MM && (pa & 15) == 0 ? 2 : (m & 1) == 0 && (pa & (2 * sizeof(TP) - 1)) == 0 ? 1 : 0;
         const int64_t ne = (int64_t)S.n * LD;
         const int64_t g0 = S.row0 * LD;
 #pragma unroll 4
@@ -291,24 +312,24 @@ k_prolong_update(const SubInfo* __restrict__ subs, const TP* __restrict__ psi, c
             const AT zs = acc + pe;              // z in the apply precision, stored so
             const double zv = widen(zs);         // (FP32 widens exactly: the iterates do not change)
             z[e] = zs;
-            if (mode != 0) {
+            if (MODE != 0) {
                 double rv = r[e];
-                const double qv = (upd || (flexible && mode == 2)) ? q[e] : 0.0;
-                if (upd) {
+                const double qv = ITER ? q[e] : 0.0;
+                if (ITER && upd) {
                     rv = fma(-alpha, qv, rv);
                     r[e] = rv;
-                    // x += alpha p here, or (x == NULL, from 8 right-hand
-                    // sides) in the next direction update, marked by xpend
-                    if (x != nullptr) x[e] = fma(alpha, p[e], x[e]);
+                    // x += alpha p here, or (from 8 right-hand sides) in the
+                    // next direction update, marked by xpend
+                    if (XUPD) x[e] = fma(alpha, p[e], x[e]);
                 }
                 v[0] = fma(rv, zv, v[0]);
                 v[1] = fma(rv, rv, v[1]);
-                if (flexible && mode == 2) v[2] = fma(zv, qv, v[2]);
+                if (FLEX) v[2] = fma(zv, qv, v[2]);
             }
         }
         __syncthreads();                 // s_ec / s_part are reused by the next subdomain
     }
-    if (mode == 0) return;
+    if (MODE == 0) return;
     int sg;
     if (!seg_reduce<4>(v, LD, R, s_out, s_scr, sg)) return;
     const int it = st->it;
@@ -317,7 +338,7 @@ k_prolong_update(const SubInfo* __restrict__ subs, const TP* __restrict__ psi, c
         const double rz = s_out[threadIdx.x];
         const double rr = s_out[LD + threadIdx.x];
         const double zq = s_out[2 * LD + threadIdx.x];
-        if (mode == 1) {
+        if (MODE == 1) {
             c.rho = rz;
             c.beta = 0.0;
             c.zq = 0.0;
@@ -341,14 +362,14 @@ k_prolong_update(const SubInfo* __restrict__ subs, const TP* __restrict__ psi, c
             } else if (rr <= st->rtol2 * c.fnorm2) {
                 c.active = 0;
                 c.beta = 0.0;
-            } else if (!flexible && !(rz > 0.0)) {
+            } else if (!FLEX && !(rz > 0.0)) {
                 // r^T M^{-1} r <= 0 in exact-arithmetic PCG: M is not SPD (the
                 // flexible variant, whose M^{-1} is applied in FP32, is only
                 // checked on its first residual, in mode 1)
                 st->status = AMS_ERR_BREAKDOWN;
                 st->done = 1;
             } else {
-                c.beta = flexible ? -zq / c.pq : rz / c.rho;
+                c.beta = FLEX ? -zq / c.pq : rz / c.rho;
             }
             c.zq = zq;
             c.rho = rz;
@@ -356,7 +377,7 @@ k_prolong_update(const SubInfo* __restrict__ subs, const TP* __restrict__ psi, c
             c.xpend = 0;   // inactive this iteration: its update (if any) was applied
         }
     }
-    if (mode != 2) return;
+    if (!ITER) return;
     if (!last_system(R, nseg)) return;
     if (threadIdx.x == 0) {
         int nact = 0;
@@ -575,14 +596,22 @@ void launch_init_norms(const LaunchCtx& L, const double* r, int nrhs) {
     AMS_DISPATCH_LD(L.ld, norms_ld, L, r, nrhs);
 }
 
-template <typename TF, typename TP, int LD>
-static void prolong_ld(const LaunchCtx& L, const ProlongArgs& a) {
-    if (L.nsub == 0) return;
-    auto kern = a.mmax > 8 ? k_prolong_update<TF, TP, LD, kMaxM> : k_prolong_update<TF, TP, LD, 8>;
+template <typename TF, typename TP, int LD, int MM>
+static void prolong_mm(const LaunchCtx& L, const ProlongArgs& a) {
+    auto kern = a.mode == 0   ? k_prolong_update<TF, TP, LD, MM, 0>
+                : a.mode == 1 ? k_prolong_update<TF, TP, LD, MM, 1>
+                : a.flexible  ? k_prolong_update<TF, TP, LD, MM, 3>
+                              : k_prolong_update<TF, TP, LD, MM, 2>;
     launch_kernel(L.pdl, kern, dim3((unsigned)L.nblk_sub), dim3(kRedThreads), 0, L.stream, L.subs, (const TP*)a.psi,
                   (const TF*)a.ec, (const TF*)a.yc, (const TF*)a.qmat, a.cref, a.gat, (const TF*)a.zf, a.r, a.q, a.x, a.p,
                   (TF*)a.z,
-                  L.red_sub, L.sc, L.st, L.nseg, a.flexible, a.mode);
+                  L.red_sub, L.sc, L.st, L.nseg);
+}
+template <typename TF, typename TP, int LD>
+static void prolong_ld(const LaunchCtx& L, const ProlongArgs& a) {
+    if (L.nsub == 0) return;
+    if (a.mmax > 8) prolong_mm<TF, TP, LD, kMaxM>(L, a);
+    else prolong_mm<TF, TP, LD, 8>(L, a);
 }
 template <typename TF, typename TP>
 static void prolong_tp(const LaunchCtx& L, const ProlongArgs& a) {
