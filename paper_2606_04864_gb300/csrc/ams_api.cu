@@ -371,6 +371,7 @@ static LaunchCtx make_ctx(ams_handle h, const RedCache& rc, const RedCache& rcs)
     L.red = layout_of(rc);
     L.red_sub = layout_of(rcs);
     L.nblk_sub = rcs.nblk;
+    L.rows = h->n_pad;
     L.nsub = h->N;
     L.sc = h->d_sc;
     L.st = h->d_st;

@@ -207,19 +207,52 @@ __device__ __forceinline__ void load_basis_row(const TP* __restrict__ pr, int m,
     }
 }
 
+// Basis row as raw 16-byte words, loaded as load_basis_row does.
+template <typename TP, int MM>
+struct RowWords {
+    static constexpr int NW = (MM * (int)sizeof(TP) + 15) / 16;
+    uint4 w[NW];
+    __device__ __forceinline__ void load(const TP* __restrict__ pr, int m, int vec) {
+        using P2 = typename std::conditional<sizeof(TP) == 2, uint32_t,
+                                             typename std::conditional<sizeof(TP) == 4, uint2, uint4>::type>::type;
+#pragma unroll
+        for (int i = 0; i < NW; ++i) w[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (vec == 2) {
+#pragma unroll
+            for (int i = 0; i < NW; ++i) w[i] = __ldg(reinterpret_cast<const uint4*>(pr) + i);
+        } else if (vec == 1) {
+#pragma unroll
+            for (int k = 0; k < MM / 2; ++k)
+                if (2 * k < m) reinterpret_cast<P2*>(w)[k] = __ldg(reinterpret_cast<const P2*>(pr) + k);
+        } else {
+#pragma unroll
+            for (int k = 0; k < MM; ++k)
+                if (k < m) reinterpret_cast<TP*>(w)[k] = pr[k];
+        }
+    }
+    __device__ __forceinline__ TP get(int k) const { return reinterpret_cast<const TP*>(w)[k]; }
+};
+
+// CH: from 8 right-hand sides (e_c comes from a launch of its own then) a block
+// takes its subdomains kChunk at a time: their rows are consecutive, so one
+// loop runs over all of them, with e_c and the basis offsets of the chunk in
+// shared memory.  One subdomain at a time costs two barriers and a drained
+// pipeline for each (8 uneven systems x 8, most of the subdomains 64 rows: 218 us
+// a launch; in chunks 178); large subdomains have no use for it, see below.
+//
 // MODE: 0 and 1 as above, 2 an iteration of PCG, 3 of flexible CG.  Bound by the
 // FP64 pipe (two thirds busy at 16 and more right-hand sides: r', three dots)
 // and the latency of its streams: the four elements a thread has in flight need
 // the loads free of branches (the mode as a run-time argument: 128^3 x 32 785
 // us, 96x80x72 x 3 78; this 735 and 72) and 64 registers, four blocks per SM
 // (two elements and six blocks 803 and 79, one and eight 834 and 79).
-template <typename TF, typename TP, int LD, int MM, int MODE>
+template <typename TF, typename TP, int LD, int MM, int MODE, bool CH>
 __global__ void __launch_bounds__(kRedThreads, 4)
 k_prolong_update(const SubInfo* __restrict__ subs, const TP* __restrict__ psi, const TF* __restrict__ ec,
                  const TF* __restrict__ yc, const TF* __restrict__ qmat, const CoarseRef* __restrict__ cref, const int32_t* __restrict__ gat,
                  const TF* __restrict__ zf, double* __restrict__ r, const double* __restrict__ q,
                  double* __restrict__ x, const double* __restrict__ p, TF* __restrict__ z, RedLayout R,
-                 CgScalars* sc, SolveState* st, int nseg) {
+                 CgScalars* sc, SolveState* st, int nseg, const int32_t* __restrict__ sub_of_row) {
     constexpr bool ITER = MODE >= 2, FLEX = MODE == 3, XUPD = ITER && LD < 8;
     using AT = typename Acc<TF>::type;
     using V4 = typename std::conditional<sizeof(TF) == 4, float4, double4>::type;
@@ -227,8 +260,14 @@ k_prolong_update(const SubInfo* __restrict__ subs, const TP* __restrict__ psi, c
     constexpr int NW = kRedThreads / 32;
     __shared__ double s_out[kRedMaxNV * kMaxLd];
     __shared__ double s_scr[kRedThreads];
-    __shared__ AT s_ec[MM * LD];
-    __shared__ AT s_part[NW * MM * LD];
+    // chunk of subdomains from 8 right-hand sides: as many e_c blocks as fit 16 KB, at most 16
+    constexpr int CH0 = 16384 / (MM * LD * (int)sizeof(AT));
+    constexpr int kChunk = !CH ? 1 : CH0 > 16 ? 16 : CH0;
+    static_assert(kChunk >= 1, "one block of e_c fits");
+    __shared__ AT s_ec[kChunk * MM * LD];
+    __shared__ AT s_part[LD < 8 ? NW * MM * LD : 1];
+    __shared__ int64_t s_psi[kChunk];                // basis offset of the subdomain's row 0, less row0 * m
+    __shared__ int s_mv[kChunk];                     // modes, and how its basis rows load
     pdl_wait();
     if (st != nullptr && st->done) return;
     pdl_trigger();
@@ -244,90 +283,156 @@ k_prolong_update(const SubInfo* __restrict__ subs, const TP* __restrict__ psi, c
     }
     double v[4] = {0.0, 0.0, 0.0, 0.0};
     const int64_t s_lo = R.blk_lo[blockIdx.x], s_hi = R.blk_lo[blockIdx.x + 1];
-    for (int64_t si = s_lo; si < s_hi; ++si) {
-        const SubInfo S = subs[si];
-        const int m = S.m;
-        const bool coarse = (ec != nullptr || qmat != nullptr) && m > 0;
-        if (coarse && ec != nullptr) {
-            // e_c computed by a separate backward-substitution launch
-            for (int i = threadIdx.x; i < MM * LD; i += kRedThreads)
-                s_ec[i] = (i < m * LD) ? (AT)ec[(int64_t)S.coff * LD + i] : AT(0);
-        } else if (coarse) {
-            // e_c rows of this subdomain: acc[k] = sum_j Q[k][j] y[gat[j]] over this thread's columns
-            const CoarseRef cr = cref[si];
-            const TF* Q = qmat + cr.q_off;
-            const int32_t* G = gat + cr.gat_off;
-            AT acc[MM];
+    auto basis_vec = [&](int64_t off, int m) {
+        const uintptr_t pa = reinterpret_cast<uintptr_t>(psi + off);
+        return m == MM && (pa & 15) == 0 ? 2 : (m & 1) == 0 && (pa & (2 * sizeof(TP) - 1)) == 0 ? 1 : 0;
+    };
+    // z = z_f + pe, the CG update and the dots of one element
+    auto finish = [&](int64_t e, AT zfv, AT pe, double rv, double qv) {
+        const AT zs = zfv + pe;              // z in the apply precision, stored so
+        const double zv = widen(zs);         // (FP32 widens exactly: the iterates do not change)
+        z[e] = zs;
+        if (MODE != 0) {
+            if (ITER && upd) {
+                rv = fma(-alpha, qv, rv);
+                r[e] = rv;
+                // x += alpha p here, or (from 8 right-hand sides) in the
+                // next direction update, marked by xpend
+                if (XUPD) x[e] = fma(alpha, p[e], x[e]);
+            }
+            v[0] = fma(rv, zv, v[0]);
+            v[1] = fma(rv, rv, v[1]);
+            if (FLEX) v[2] = fma(zv, qv, v[2]);
+        }
+    };
+    if constexpr (CH) {
+        using Row = RowWords<TP, MM>;
+        constexpr int U = Row::NW * 4 > 16 ? 1 : Row::NW * 4 > 8 ? 2 : 4;   // elements in flight
+        const bool coarse = ec != nullptr;
+        for (int64_t c0 = s_lo; c0 < s_hi; c0 += kChunk) {
+            const int nsub = (int)(s_hi - c0 < kChunk ? s_hi - c0 : kChunk);
+            if (threadIdx.x < nsub) {
+                const SubInfo S = subs[c0 + threadIdx.x];
+                s_psi[threadIdx.x] = S.psi_off - S.row0 * S.m;
+                s_mv[threadIdx.x] = S.m * 4 + basis_vec(S.psi_off, S.m);
+            }
+            if (coarse)
+                for (int i = threadIdx.x; i < nsub * MM * LD; i += kRedThreads) {
+                    const SubInfo* S = subs + c0 + i / (MM * LD);
+                    const int k = i % (MM * LD);
+                    s_ec[i] = k < S->m * LD ? (AT)ec[S->coff * LD + k] : AT(0);
+                }
+            const int64_t e0 = subs[c0].row0 * LD;
+            const int64_t e1 = (subs[c0 + nsub - 1].row0 + subs[c0 + nsub - 1].n) * LD;
+            __syncthreads();
+            for (int64_t eb = e0 + threadIdx.x; eb < e1; eb += U * kRedThreads) {
+                AT zv[U];
+                double rv[U], qv[U];
+                int si[U];
+                Row row[U];
 #pragma unroll
-            for (int k = 0; k < MM; ++k) acc[k] = AT(0);
-            for (int c4 = cg; 4 * c4 < cr.K; c4 += NCG) {
-                const int j0 = 4 * c4;
-                AT yv[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    yv[e] = AT(0);
-                    if (j0 + e < cr.K) {
-                        const int gi = __ldg(G + j0 + e);
-                        if (AMS_COARSE_OK(gi, 2)) yv[e] = (AT)yc[(int64_t)gi * LD + rhs];
+                for (int u = 0; u < U; ++u) {
+                    const int64_t e = eb + u * kRedThreads;
+                    zv[u] = AT(0);
+                    rv[u] = qv[u] = 0.0;
+                    si[u] = 0;
+                    if (e < e1) {
+                        if (coarse) si[u] = (int)(__ldg(sub_of_row + e / LD) - c0);
+                        zv[u] = (AT)zf[e];
+                        if (MODE != 0) rv[u] = r[e];
+                        if (ITER) qv[u] = q[e];
                     }
                 }
+                if (coarse)
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int64_t e = eb + u * kRedThreads;
+                        const int mv = s_mv[si[u]], m = mv >> 2;
+                        if (e < e1) row[u].load(psi + s_psi[si[u]] + e / LD * m, m, mv & 3);
+                    }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int64_t e = eb + u * kRedThreads;
+                    if (e >= e1) break;
+                    AT pe = AT(0);
+                    if (coarse)
+#pragma unroll
+                        for (int k = 0; k < MM; ++k)
+                            pe += (AT)to_d(row[u].get(k)) * s_ec[(si[u] * MM + k) * LD + rhs];
+                    finish(e, zv[u], pe, rv[u], qv[u]);
+                }
+            }
+            __syncthreads();                 // the chunk's tables are reused by the next
+        }
+    } else {
+        for (int64_t si = s_lo; si < s_hi; ++si) {
+            const SubInfo S = subs[si];
+            const int m = S.m;
+            const bool coarse = (ec != nullptr || qmat != nullptr) && m > 0;
+            if (coarse && ec != nullptr) {
+                // e_c computed by a separate backward-substitution launch
+                for (int i = threadIdx.x; i < MM * LD; i += kRedThreads)
+                    s_ec[i] = (i < m * LD) ? (AT)ec[(int64_t)S.coff * LD + i] : AT(0);
+            } else if (coarse) {
+                // e_c rows of this subdomain: acc[k] = sum_j Q[k][j] y[gat[j]] over this thread's columns
+                const CoarseRef cr = cref[si];
+                const TF* Q = qmat + cr.q_off;
+                const int32_t* G = gat + cr.gat_off;
+                AT acc[MM];
+#pragma unroll
+                for (int k = 0; k < MM; ++k) acc[k] = AT(0);
+                for (int c4 = cg; 4 * c4 < cr.K; c4 += NCG) {
+                    const int j0 = 4 * c4;
+                    AT yv[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        yv[e] = AT(0);
+                        if (j0 + e < cr.K) {
+                            const int gi = __ldg(G + j0 + e);
+                            if (AMS_COARSE_OK(gi, 2)) yv[e] = (AT)yc[(int64_t)gi * LD + rhs];
+                        }
+                    }
+#pragma unroll
+                    for (int k = 0; k < MM; ++k) {
+                        if (k < m) {
+                            const V4 qv = *reinterpret_cast<const V4*>(Q + (int64_t)k * cr.ldm + j0);
+                            acc[k] += (AT)qv.x * yv[0] + (AT)qv.y * yv[1] + (AT)qv.z * yv[2] + (AT)qv.w * yv[3];
+                        }
+                    }
+                }
+                // sum over column groups: lanes of a warp with the same rhs, then warps in order
 #pragma unroll
                 for (int k = 0; k < MM; ++k) {
-                    if (k < m) {
-                        const V4 qv = *reinterpret_cast<const V4*>(Q + (int64_t)k * cr.ldm + j0);
-                        acc[k] += (AT)qv.x * yv[0] + (AT)qv.y * yv[1] + (AT)qv.z * yv[2] + (AT)qv.w * yv[3];
-                    }
+                    AT a = acc[k];
+                    for (int off = 16; off >= LD; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+                    if (lane < LD) s_part[(warp * MM + k) * LD + lane] = a;
                 }
-            }
-            // sum over column groups: lanes of a warp with the same rhs, then warps in order
-#pragma unroll
-            for (int k = 0; k < MM; ++k) {
-                AT a = acc[k];
-                for (int off = 16; off >= LD; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
-                if (lane < LD) s_part[(warp * MM + k) * LD + lane] = a;
+                __syncthreads();
+                for (int i = threadIdx.x; i < MM * LD; i += kRedThreads) {
+                    AT a = AT(0);
+                    for (int w = 0; w < NW; ++w) a += s_part[w * MM * LD + i];
+                    s_ec[i] = a;
+                }
             }
             __syncthreads();
-            for (int i = threadIdx.x; i < MM * LD; i += kRedThreads) {
-                AT a = AT(0);
-                for (int w = 0; w < NW; ++w) a += s_part[w * MM * LD + i];
-                s_ec[i] = a;
-            }
-        }
-        __syncthreads();
-        const uintptr_t pa = reinterpret_cast<uintptr_t>(psi + S.psi_off);
-        const int vec = m == MM && (pa & 15) == 0 ? 2 : (m & 1) == 0 && (pa & (2 * sizeof(TP) - 1)) == 0 ? 1 : 0;
-        const int64_t ne = (int64_t)S.n * LD;
-        const int64_t g0 = S.row0 * LD;
+            const int vec = basis_vec(S.psi_off, m);
+            const int64_t ne = (int64_t)S.n * LD;
+            const int64_t g0 = S.row0 * LD;
 #pragma unroll 4
-        for (int64_t le = threadIdx.x; le < ne; le += kRedThreads) {
-            const int64_t e = g0 + le;
-            AT acc = (AT)zf[e];
-            AT pe = AT(0);
-            if (coarse) {
-                TP pv[MM];
-                load_basis_row<TP, MM>(psi + S.psi_off + (le / LD) * m, m, vec, pv);
+            for (int64_t le = threadIdx.x; le < ne; le += kRedThreads) {
+                const int64_t e = g0 + le;
+                AT acc = (AT)zf[e];
+                AT pe = AT(0);
+                if (coarse) {
+                    TP pv[MM];
+                    load_basis_row<TP, MM>(psi + S.psi_off + (le / LD) * m, m, vec, pv);
 #pragma unroll
-                for (int k = 0; k < MM; ++k) pe += (AT)to_d(pv[k]) * s_ec[k * LD + rhs];
-            }
-            const AT zs = acc + pe;              // z in the apply precision, stored so
-            const double zv = widen(zs);         // (FP32 widens exactly: the iterates do not change)
-            z[e] = zs;
-            if (MODE != 0) {
-                double rv = r[e];
-                const double qv = ITER ? q[e] : 0.0;
-                if (ITER && upd) {
-                    rv = fma(-alpha, qv, rv);
-                    r[e] = rv;
-                    // x += alpha p here, or (from 8 right-hand sides) in the
-                    // next direction update, marked by xpend
-                    if (XUPD) x[e] = fma(alpha, p[e], x[e]);
+                    for (int k = 0; k < MM; ++k) pe += (AT)to_d(pv[k]) * s_ec[k * LD + rhs];
                 }
-                v[0] = fma(rv, zv, v[0]);
-                v[1] = fma(rv, rv, v[1]);
-                if (FLEX) v[2] = fma(zv, qv, v[2]);
+                finish(e, acc, pe, MODE != 0 ? r[e] : 0.0, ITER ? q[e] : 0.0);
             }
+            __syncthreads();                 // s_ec / s_part are reused by the next subdomain
         }
-        __syncthreads();                 // s_ec / s_part are reused by the next subdomain
     }
     if (MODE == 0) return;
     int sg;
@@ -596,16 +701,28 @@ void launch_init_norms(const LaunchCtx& L, const double* r, int nrhs) {
     AMS_DISPATCH_LD(L.ld, norms_ld, L, r, nrhs);
 }
 
-template <typename TF, typename TP, int LD, int MM>
-static void prolong_mm(const LaunchCtx& L, const ProlongArgs& a) {
-    auto kern = a.mode == 0   ? k_prolong_update<TF, TP, LD, MM, 0>
-                : a.mode == 1 ? k_prolong_update<TF, TP, LD, MM, 1>
-                : a.flexible  ? k_prolong_update<TF, TP, LD, MM, 3>
-                              : k_prolong_update<TF, TP, LD, MM, 2>;
+template <typename TF, typename TP, int LD, int MM, bool CH>
+static void prolong_ch(const LaunchCtx& L, const ProlongArgs& a) {
+    auto kern = a.mode == 0   ? k_prolong_update<TF, TP, LD, MM, 0, CH>
+                : a.mode == 1 ? k_prolong_update<TF, TP, LD, MM, 1, CH>
+                : a.flexible  ? k_prolong_update<TF, TP, LD, MM, 3, CH>
+                              : k_prolong_update<TF, TP, LD, MM, 2, CH>;
     launch_kernel(L.pdl, kern, dim3((unsigned)L.nblk_sub), dim3(kRedThreads), 0, L.stream, L.subs, (const TP*)a.psi,
                   (const TF*)a.ec, (const TF*)a.yc, (const TF*)a.qmat, a.cref, a.gat, (const TF*)a.zf, a.r, a.q, a.x, a.p,
                   (TF*)a.z,
-                  L.red_sub, L.sc, L.st, L.nseg);
+                  L.red_sub, L.sc, L.st, L.nseg, L.sub_of_row);
+}
+// In chunks up to 2048 elements a subdomain on average, two passes of a block
+// over it.  One subdomain at a time / in chunks, us a launch: 1430 elements (the
+// uneven systems) 218 / 178, 2048 (512^2 in 16 x 16 blocks x 8) 59 / 57.6; 3650
+// (77^3 x 8) 84 / 86, 4096 (64^3 x 8) 53 / 55, 8192 (96^3 x 16) 200 / 204, where
+// the row's subdomain is one more load before the basis.  FP64 62 / 65 at 2900.
+template <typename TF, typename TP, int LD, int MM>
+static void prolong_mm(const LaunchCtx& L, const ProlongArgs& a) {
+    if constexpr (LD >= 8 && sizeof(TF) == 4) {
+        if (L.rows * LD <= 2048 * (int64_t)L.nsub) return prolong_ch<TF, TP, LD, MM, true>(L, a);
+    }
+    prolong_ch<TF, TP, LD, MM, false>(L, a);
 }
 template <typename TF, typename TP, int LD>
 static void prolong_ld(const LaunchCtx& L, const ProlongArgs& a) {

@@ -38,6 +38,7 @@ struct LaunchCtx {
     RedLayout red_sub;       // blocks of consecutive subdomains
     int64_t nblk_sub;        // blocks of red_sub
     int nsub;                // subdomains
+    int64_t rows;            // internal rows (padding included)
     CgScalars* sc;           // [nseg][ld]
     SolveState* st;
     bool pdl;                // solve-loop kernels: programmatic dependent launch
