@@ -16,6 +16,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "ams_internal.h"
+#include "host_parallel.h"
 #include "kernels.cuh"
 #include "launch.h"
 
@@ -692,24 +693,15 @@ static ams_status setup_coarse(ams_handle h, const std::vector<SysInput>& inputs
     const double t0 = now_s();
     // coarse layout per system: ND order of the subdomain graph
     int64_t coff = 0;
+    std::vector<std::vector<int64_t>> sub_adj_ptr(h->nsys);
+    std::vector<std::vector<int32_t>> sub_adj(h->nsys);
     for (int s = 0; s < h->nsys; ++s) {
         SystemHost& S = h->sys[s];
         const SysInput& in = inputs[s];
         const int32_t N = S.nparts;
-        std::vector<std::vector<int32_t>> nb(N);
-        for (int64_t i = 0; i < S.n; ++i)
-            for (int64_t e = in.A.rowptr[i]; e < in.A.rowptr[i + 1]; ++e) {
-                const int32_t a = in.part[i], b = in.part[in.A.colind[e]];
-                if (a != b) nb[a].push_back(b);
-            }
-        std::vector<int64_t> adj_ptr(N + 1, 0);
-        std::vector<int32_t> adj;
-        for (int32_t a = 0; a < N; ++a) {
-            std::sort(nb[a].begin(), nb[a].end());
-            nb[a].erase(std::unique(nb[a].begin(), nb[a].end()), nb[a].end());
-            adj.insert(adj.end(), nb[a].begin(), nb[a].end());
-            adj_ptr[a + 1] = adj.size();
-        }
+        std::vector<int64_t>& adj_ptr = sub_adj_ptr[s];
+        std::vector<int32_t>& adj = sub_adj[s];
+        AMS_TRY(subdomain_graph(in.A, in.part.data(), N, S.perm, S.sub_ptr, adj_ptr, adj));
         std::vector<int32_t> w(N);
         for (int32_t a = 0; a < N; ++a) w[a] = h->h_subs[S.sub0 + a].m;
         nested_dissection(N, adj_ptr, adj, w, 96, S.nodes);
@@ -737,18 +729,12 @@ static ams_status setup_coarse(ams_handle h, const std::vector<SysInput>& inputs
     int max_nbr = 1;
     for (int s = 0; s < h->nsys; ++s) {
         const SystemHost& S = h->sys[s];
-        const SysInput& in = inputs[s];
-        std::vector<std::vector<int32_t>> nb(S.nparts);
-        for (int64_t i = 0; i < S.n; ++i)
-            for (int64_t e = in.A.rowptr[i]; e < in.A.rowptr[i + 1]; ++e)
-                nb[in.part[i]].push_back(S.sub0 + in.part[in.A.colind[e]]);
         for (int32_t a = 0; a < S.nparts; ++a) {
-            auto& v = nb[a];
-            std::sort(v.begin(), v.end());
-            v.erase(std::unique(v.begin(), v.end()), v.end());
-            nbr.insert(nbr.end(), v.begin(), v.end());
+            const size_t first = nbr.size();
+            for (int64_t k = sub_adj_ptr[s][a]; k < sub_adj_ptr[s][a + 1]; ++k) nbr.push_back(S.sub0 + sub_adj[s][k]);
+            nbr.insert(std::lower_bound(nbr.begin() + first, nbr.end(), S.sub0 + a), S.sub0 + a);
             nbr_ptr[S.sub0 + a + 1] = nbr.size();
-            max_nbr = std::max(max_nbr, (int)v.size());
+            max_nbr = std::max(max_nbr, (int)(nbr.size() - first));
         }
     }
     if (max_nbr > 256) {
@@ -1051,62 +1037,78 @@ static ams_status setup_impl(int32_t nsys, const ams_system_desc* systems, const
     }
     // index maps, internal CSR, subdomain descriptors
     std::vector<int64_t> int_row(h->n_total), irp(h->n_pad + 1, 0);
-    std::vector<int32_t> sub_of_row(h->n_pad, -1), icol;
-    std::vector<double> ival;
-    icol.reserve(h->nnz_total);
-    ival.reserve(h->nnz_total);
+    std::vector<int32_t> sub_of_row(h->n_pad, -1);
     h->h_subs.resize(h->N);
-    std::vector<std::pair<int32_t, double>> rowbuf;
-    std::vector<std::pair<int32_t, int64_t>> rowsrc;   // (internal col, caller entry)
-    std::vector<int64_t> ientry_src;                    // internal CSR entry -> caller entry
-    ientry_src.reserve(h->nnz_total);
-    int64_t rp = 0;
+    std::vector<int32_t> icol(h->nnz_total);
+    std::vector<double> ival(h->nnz_total);
+    std::vector<int64_t> ientry_src(h->nnz_total);      // internal CSR entry -> caller entry
     for (int s = 0; s < nsys; ++s) {
         SystemHost& S = h->sys[s];
         const HostCSR& A = inputs[s].A;
         std::vector<int64_t> iperm(S.n);
         for (int64_t k = 0; k < S.n; ++k) iperm[S.perm[k]] = k;
         for (int64_t g = 0; g < S.n; ++g) int_row[S.caller0 + g] = S.row0 + iperm[g];
+        // subdomain descriptors and row lengths (rows of a subdomain are consecutive)
+        parallel_chunks(S.nparts, 64, [&](int64_t a0, int64_t a1, int) {
+            for (int64_t a = a0; a < a1; ++a) {
+                SubInfo& I = h->h_subs[S.sub0 + a];
+                I = SubInfo{};
+                I.row0 = S.row0 + S.sub_ptr[a];
+                I.n = (int32_t)(S.sub_ptr[a + 1] - S.sub_ptr[a]);
+                I.nb = (I.n + 31) / 32;
+                I.seg = s;
+                I.m = 0;
+                int64_t bw = 0;
+                for (int64_t k = S.sub_ptr[a]; k < S.sub_ptr[a + 1]; ++k) {
+                    sub_of_row[S.row0 + k] = (int32_t)(S.sub0 + a);
+                    const int64_t g = S.perm[k];
+                    irp[S.row0 + k + 1] = A.rowptr[g + 1] - A.rowptr[g];
+                    for (int64_t e = A.rowptr[g]; e < A.rowptr[g + 1]; ++e) {
+                        const int64_t kk = iperm[A.colind[e]];
+                        if (kk >= S.sub_ptr[a] && kk < k) bw = std::max(bw, k - kk);
+                    }
+                }
+                I.c = (int32_t)std::max<int64_t>(1, (bw + 31) / 32);
+            }
+        });
         for (int32_t a = 0; a < S.nparts; ++a) {
-            SubInfo& I = h->h_subs[S.sub0 + a];
-            I = SubInfo{};
-            I.row0 = S.row0 + S.sub_ptr[a];
-            I.n = (int32_t)(S.sub_ptr[a + 1] - S.sub_ptr[a]);
-            I.nb = (I.n + 31) / 32;
+            const SubInfo& I = h->h_subs[S.sub0 + a];
             h->nbmax = std::max(h->nbmax, (int)I.nb);
-            I.seg = s;
-            I.m = 0;
-            int64_t bw = 0;
-            for (int64_t k = S.sub_ptr[a]; k < S.sub_ptr[a + 1]; ++k) {
-                sub_of_row[S.row0 + k] = S.sub0 + a;
-                const int64_t g = S.perm[k];
-                for (int64_t e = A.rowptr[g]; e < A.rowptr[g + 1]; ++e) {
-                    const int64_t kk = iperm[A.colind[e]];
-                    if (kk >= S.sub_ptr[a] && kk < k) bw = std::max(bw, k - kk);
+            h->cmax = std::max(h->cmax, (int)I.c);
+        }
+        for (int64_t k = 0; k < S.npad; ++k) irp[S.row0 + k + 1] += irp[S.row0 + k];
+        // entries of every row by internal column
+        bool oom[kMaxChunks] = {};
+        const int nchunk = parallel_chunks(S.n, 8192, [&](int64_t k0, int64_t k1, int chunk) {
+            std::pair<int32_t, int64_t> few[64];        // (internal col, caller entry)
+            std::vector<std::pair<int32_t, int64_t>> many;
+            for (int64_t k = k0; k < k1; ++k) {
+                const int64_t b = A.rowptr[S.perm[k]], len = A.rowptr[S.perm[k] + 1] - b, o = irp[S.row0 + k];
+                std::pair<int32_t, int64_t>* v = few;
+                if (len > 64) {
+                    try {
+                        many.resize(len);
+                    } catch (const std::bad_alloc&) {
+                        oom[chunk] = true;
+                        return;
+                    }
+                    v = many.data();
+                }
+                for (int64_t j = 0; j < len; ++j) v[j] = {(int32_t)(S.row0 + iperm[A.colind[b + j]]), b + j};
+                std::sort(v, v + len);
+                for (int64_t j = 0; j < len; ++j) {
+                    icol[o + j] = v[j].first;
+                    ival[o + j] = A.vals[v[j].second];
+                    ientry_src[o + j] = S.caller_nnz0 + v[j].second;
                 }
             }
-            I.c = (int32_t)std::max<int64_t>(1, (bw + 31) / 32);
-            h->cmax = std::max(h->cmax, I.c);
-        }
-        for (int64_t k = 0; k < S.npad; ++k) {
-            irp[S.row0 + k] = rp;
-            if (k < S.n) {
-                const int64_t g = S.perm[k];
-                rowsrc.clear();
-                for (int64_t e = A.rowptr[g]; e < A.rowptr[g + 1]; ++e)
-                    rowsrc.push_back({(int32_t)(S.row0 + iperm[A.colind[e]]), S.caller_nnz0 + e});
-                std::sort(rowsrc.begin(), rowsrc.end());
-                for (auto& pr : rowsrc) {
-                    icol.push_back(pr.first);
-                    const int64_t ce = pr.second - S.caller_nnz0;
-                    ival.push_back(A.vals[ce]);
-                    ientry_src.push_back(pr.second);
-                }
-                rp += (int64_t)rowsrc.size();
+        });
+        for (int c = 0; c < nchunk; ++c)
+            if (oom[c]) {
+                set_error("out of host memory for a matrix row");
+                return AMS_ERR_OOM;
             }
-        }
     }
-    irp[h->n_pad] = rp;
     {
         std::vector<int32_t> order;
         for (int c = 1; c <= h->cmax; ++c) {
@@ -1140,32 +1142,36 @@ static ams_status setup_impl(int32_t nsys, const ams_system_desc* systems, const
     // SELL-32 layout of the internal matrix
     const int64_t nslices = h->n_pad / 32;
     std::vector<int64_t> sell_ptr(nslices + 1, 0);
-    for (int64_t sl = 0; sl < nslices; ++sl) {
-        int64_t w = 0;
-        for (int l = 0; l < 32; ++l) w = std::max(w, irp[sl * 32 + l + 1] - irp[sl * 32 + l]);
-        sell_ptr[sl + 1] = sell_ptr[sl] + 32 * w;
-    }
+    parallel_chunks(nslices, 512, [&](int64_t s0, int64_t s1, int) {
+        for (int64_t sl = s0; sl < s1; ++sl) {
+            int64_t w = 0;
+            for (int l = 0; l < 32; ++l) w = std::max(w, irp[sl * 32 + l + 1] - irp[sl * 32 + l]);
+            sell_ptr[sl + 1] = 32 * w;
+        }
+    });
+    for (int64_t sl = 0; sl < nslices; ++sl) sell_ptr[sl + 1] += sell_ptr[sl];
     std::vector<int32_t> sell_col(sell_ptr[nslices]);
     std::vector<double> sell_val(sell_ptr[nslices], 0.0);
     std::vector<int64_t> sell_pos(h->nnz_total, 0);
-    for (int64_t sl = 0; sl < nslices; ++sl) {
-        const int64_t w = (sell_ptr[sl + 1] - sell_ptr[sl]) / 32;
-        for (int l = 0; l < 32; ++l) {
-            const int64_t r = sl * 32 + l;
-            const int64_t len = irp[r + 1] - irp[r];
-            for (int64_t j = 0; j < w; ++j) {
-                const int64_t o = sell_ptr[sl] + 32 * j + l;
-                if (j < len) {
-                    sell_col[o] = icol[irp[r] + j];
-                    sell_val[o] = ival[irp[r] + j];
-                    sell_pos[ientry_src[irp[r] + j]] = o;
-                } else {
-                    sell_col[o] = (int32_t)r;
-                    sell_val[o] = 0.0;
+    parallel_chunks(nslices, 512, [&](int64_t s0, int64_t s1, int) {
+        for (int64_t sl = s0; sl < s1; ++sl) {
+            const int64_t w = (sell_ptr[sl + 1] - sell_ptr[sl]) / 32;
+            for (int l = 0; l < 32; ++l) {
+                const int64_t r = sl * 32 + l;
+                const int64_t len = irp[r + 1] - irp[r];
+                for (int64_t j = 0; j < w; ++j) {
+                    const int64_t o = sell_ptr[sl] + 32 * j + l;
+                    if (j < len) {
+                        sell_col[o] = icol[irp[r] + j];
+                        sell_val[o] = ival[irp[r] + j];
+                        sell_pos[ientry_src[irp[r] + j]] = o;
+                    } else {
+                        sell_col[o] = (int32_t)r;
+                    }
                 }
             }
         }
-    }
+    });
     ams_handle H = h.get();
     AMS_TRY(upload(H, &h->d_int_row, int_row));
     AMS_TRY(upload(H, &h->d_sub_of_row, sub_of_row));

@@ -157,6 +157,11 @@ void build_index_maps(int64_t n, const int32_t* part, int32_t nparts,
                       std::vector<int64_t>& perm, std::vector<int64_t>& iperm,
                       std::vector<int64_t>& sub_ptr);
 
+// Neighbouring subdomains of every subdomain (no self loops, ascending), as CSR.
+ams_status subdomain_graph(const HostCSR& A, const int32_t* part, int32_t nparts, const std::vector<int64_t>& perm,
+                           const std::vector<int64_t>& sub_ptr, std::vector<int64_t>& adj_ptr,
+                           std::vector<int32_t>& adj);
+
 // Nested-dissection tree of the coarse (subdomain) graph.
 struct NDNode {
     std::vector<int32_t> subs;   // subdomains of this node, in coarse order

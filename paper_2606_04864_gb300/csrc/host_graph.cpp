@@ -5,11 +5,13 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <new>
 #include <numeric>
 #include <string>
 #include <vector>
 
 #include "ams_internal.h"
+#include "host_parallel.h"
 
 namespace ams {
 
@@ -28,53 +30,57 @@ ams_status validate_system(const HostCSR& A, const int32_t* part, int32_t nparts
         set_error("rowptr[0] must be 0");
         return AMS_ERR_INVALID_ARG;
     }
-    for (int64_t i = 0; i < n; ++i) {
-        const int64_t b = A.rowptr[i], e = A.rowptr[i + 1];
-        if (e < b) {
-            std::snprintf(buf, sizeof buf, "rowptr decreases at row %lld", (long long)i);
-            set_error(buf);
-            return AMS_ERR_INVALID_ARG;
-        }
-        bool diag = false;
-        for (int64_t t = b; t < e; ++t) {
-            const int32_t c = A.colind[t];
-            if (c < 0 || c >= n) {
-                std::snprintf(buf, sizeof buf, "column index out of range in row %lld", (long long)i);
-                set_error(buf);
-                return AMS_ERR_INVALID_ARG;
-            }
-            if (t > b && A.colind[t - 1] >= c) {
-                std::snprintf(buf, sizeof buf, "columns not strictly ascending in row %lld", (long long)i);
-                set_error(buf);
-                return AMS_ERR_INVALID_ARG;
-            }
-            if (c == i) {
-                diag = true;
-                if (!(A.vals[t] > 0.0)) {
-                    std::snprintf(buf, sizeof buf, "non-positive diagonal in row %lld", (long long)i);
-                    set_error(buf);
-                    return AMS_ERR_NOT_SPD;
+    // rows 0 .. up - 1 have increasing pointers; a row that has not ends the checks there
+    int64_t up = 0;
+    while (up < n && A.rowptr[up + 1] >= A.rowptr[up]) ++up;
+    const int64_t nnz = A.rowptr[n];
+    // Rows are independent: checked in chunks, the first chunk with an error
+    // (its first row) reports it, as one pass over the rows would.
+    struct Fault {
+        ams_status st = AMS_OK;
+        char msg[96] = "";
+    };
+    Fault fault[kMaxChunks];
+    const int nchunk = parallel_chunks(up, 8192, [&](int64_t i0, int64_t i1, int chunk) {
+        Fault& F = fault[chunk];
+        auto fail = [&](ams_status st, const char* fmt, long long i, int c) {
+            F.st = st;
+            std::snprintf(F.msg, sizeof F.msg, fmt, i, c);
+        };
+        for (int64_t i = i0; i < i1; ++i) {
+            const int64_t b = A.rowptr[i], e = std::min(A.rowptr[i + 1], nnz);
+            bool diag = false;
+            for (int64_t t = b; t < e; ++t) {
+                const int32_t c = A.colind[t];
+                if (c < 0 || c >= n) return fail(AMS_ERR_INVALID_ARG, "column index out of range in row %lld", i, 0);
+                if (t > b && A.colind[t - 1] >= c)
+                    return fail(AMS_ERR_INVALID_ARG, "columns not strictly ascending in row %lld", i, 0);
+                if (c == i) {
+                    diag = true;
+                    if (!(A.vals[t] > 0.0)) return fail(AMS_ERR_NOT_SPD, "non-positive diagonal in row %lld", i, 0);
                 }
+                if (!std::isfinite(A.vals[t])) return fail(AMS_ERR_INVALID_ARG, "non-finite matrix value", i, 0);
+                // symmetric partner (c, i) with the identical value
+                if (A.rowptr[c + 1] < A.rowptr[c]) continue;   // reported below
+                const int64_t pb = std::min(std::max<int64_t>(A.rowptr[c], 0), std::max<int64_t>(nnz, 0));
+                const int64_t pe = std::max(pb, std::min(A.rowptr[c + 1], nnz));
+                const int32_t* ce = A.colind.data() + pe;
+                const int32_t* f = std::lower_bound(A.colind.data() + pb, ce, (int32_t)i);
+                if (f == ce || *f != i || A.vals[f - A.colind.data()] != A.vals[t])
+                    return fail(AMS_ERR_INVALID_ARG, "matrix not symmetric at (%lld, %d)", i, c);
             }
-            if (!std::isfinite(A.vals[t])) {
-                set_error("non-finite matrix value");
-                return AMS_ERR_INVALID_ARG;
-            }
-            // symmetric partner (c, i) with the identical value
-            const int32_t* cb = A.colind.data() + A.rowptr[c];
-            const int32_t* ce = A.colind.data() + A.rowptr[c + 1];
-            const int32_t* f = std::lower_bound(cb, ce, (int32_t)i);
-            if (f == ce || *f != i || A.vals[A.rowptr[c] + (f - cb)] != A.vals[t]) {
-                std::snprintf(buf, sizeof buf, "matrix not symmetric at (%lld, %d)", (long long)i, c);
-                set_error(buf);
-                return AMS_ERR_INVALID_ARG;
-            }
+            if (!diag) return fail(AMS_ERR_INVALID_ARG, "missing diagonal in row %lld", i, 0);
         }
-        if (!diag) {
-            std::snprintf(buf, sizeof buf, "missing diagonal in row %lld", (long long)i);
-            set_error(buf);
-            return AMS_ERR_INVALID_ARG;
+    });
+    for (int c = 0; c < nchunk; ++c)
+        if (fault[c].st != AMS_OK) {
+            set_error(fault[c].msg);
+            return fault[c].st;
         }
+    if (up < n) {
+        std::snprintf(buf, sizeof buf, "rowptr decreases at row %lld", (long long)up);
+        set_error(buf);
+        return AMS_ERR_INVALID_ARG;
     }
     std::vector<int64_t> cnt(nparts, 0);
     for (int64_t i = 0; i < n; ++i) {
@@ -109,6 +115,47 @@ void build_index_maps(int64_t n, const int32_t* part, int32_t nparts,
         perm[k] = i;
         iperm[i] = k;
     }
+}
+
+// Neighbouring subdomains (without itself, ascending) of every subdomain, as
+// a CSR graph.
+ams_status subdomain_graph(const HostCSR& A, const int32_t* part, int32_t nparts, const std::vector<int64_t>& perm,
+                           const std::vector<int64_t>& sub_ptr, std::vector<int64_t>& adj_ptr,
+                           std::vector<int32_t>& adj) {
+    adj_ptr.assign(nparts + 1, 0);
+    std::vector<int32_t> lists[kMaxChunks];
+    bool oom[kMaxChunks] = {};
+    const int nchunk = parallel_chunks(nparts, 64, [&](int64_t a0, int64_t a1, int chunk) {
+        try {
+            std::vector<int32_t> seen(nparts, -1);
+            auto& list = lists[chunk];
+            for (int64_t a = a0; a < a1; ++a) {
+                const size_t first = list.size();
+                for (int64_t k = sub_ptr[a]; k < sub_ptr[a + 1]; ++k)
+                    for (int64_t e = A.rowptr[perm[k]]; e < A.rowptr[perm[k] + 1]; ++e) {
+                        const int32_t b = part[A.colind[e]];
+                        if (b != a && seen[b] != a) {
+                            seen[b] = (int32_t)a;
+                            list.push_back(b);
+                        }
+                    }
+                std::sort(list.begin() + first, list.end());
+                adj_ptr[a + 1] = (int64_t)(list.size() - first);
+            }
+        } catch (const std::bad_alloc&) {
+            oom[chunk] = true;
+        }
+    });
+    for (int c = 0; c < nchunk; ++c)
+        if (oom[c]) {
+            set_error("out of host memory for the subdomain graph");
+            return AMS_ERR_OOM;
+        }
+    for (int32_t a = 0; a < nparts; ++a) adj_ptr[a + 1] += adj_ptr[a];
+    adj.clear();
+    adj.reserve(adj_ptr[nparts]);
+    for (int c = 0; c < nchunk; ++c) adj.insert(adj.end(), lists[c].begin(), lists[c].end());
+    return AMS_OK;
 }
 
 // ---------------------------------------------------------------------------
