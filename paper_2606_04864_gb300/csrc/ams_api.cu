@@ -562,7 +562,7 @@ static ams_status setup_eigen(ams_handle h, const int64_t* d_rowptr, const int32
     SubInfo* d_esubs = nullptr;
     AMS_TRY(upload(h, &d_esubs, esubs));
     LocalSolveArgs la{h->stream, h->N, d_esubs, ResidIn{d_X, nullptr, nullptr}, d_S, P, h->cmax, 0, nullptr, false,
-                      0, P};
+                      0, P, h->num_sms};
     const int maxit = h->opt.eig_maxit > 0 ? h->opt.eig_maxit : 300;
     const double tol = h->opt.eig_tol > 0 ? h->opt.eig_tol : 1e-13;
     std::vector<double> res(2 * (size_t)h->N);   // per subdomain: residual, then the spread of its shifted Ritz values
@@ -1380,7 +1380,8 @@ static ams_status launch_local(ams_handle h, int ld, const ResidIn& in, bool wit
         AMS_CUDA_TRY(launch_local_tma(a, h->prec, h->d_psi, h->d_psif, h->d_zf, coarse ? h->d_rc : nullptr));
     } else {
         LocalSolveArgs la{h->stream, h->N, h->d_subs, in, nullptr, ld, h->cmax, std::max(1, h->mmax),
-                          with_state ? h->d_st : nullptr, h->use_pdl, h->tune[ld].depth, h->ncols};
+                          with_state ? h->d_st : nullptr, h->use_pdl, h->tune[ld].depth, h->ncols,
+                          h->num_sms};
         AMS_CUDA_TRY(launch_local_solve(la, (const double*)h->d_fac, (const double*)h->d_psi, (double*)h->d_zf,
                                         coarse ? (double*)h->d_rc : nullptr));
     }

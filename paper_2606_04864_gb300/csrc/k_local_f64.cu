@@ -321,8 +321,257 @@ k_local_f64(const SubInfo* __restrict__ subs, const double* __restrict__ fac, co
     }
 }
 
+// One to four right-hand sides on many subdomains of one tile a block row: a
+// lane per row (forward) or column (backward), NR columns a warp, with the
+// triangles' other halves masked.  64 multiply-adds a lane and tile pair where
+// row pairs take 33, but no lane idles and no partial sums are added up across
+// lanes, which with few columns and one tile costs more FP64 instructions than
+// the masks.  Left-looking in both sweeps: step K of the backward one needs
+// block rows K .. K + c.
+template <int NR, int MM>
+__global__ void k_local_f64_rows(const SubInfo* __restrict__ subs, const double* __restrict__ fac,
+                              const double* __restrict__ rin, const double* __restrict__ qin,
+                              const CgScalars* __restrict__ csc, const double* __restrict__ rowscale,
+                              double* __restrict__ zf, const double* __restrict__ psi, double* __restrict__ rc,
+                              int ld, int cmax, int depth, const SolveState* st) {
+    pdl_wait();
+    if (st != nullptr && st->done) return;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const SubInfo S = subs[blockIdx.x];
+    const int c = S.c, nb = S.nb, n = S.n;
+    const int D = depth;                                       // block rows in flight
+    const int nbuf = c + D + 1;
+    const int64_t brs = blockrow_elems(c);
+    const int64_t brs_max = blockrow_elems(cmax);
+    double* bufs = (double*)smem_raw;                                  // (cmax+D+1) * brs_max
+    double* ring = bufs + (int64_t)(cmax + D + 1) * brs_max;       // (cmax+1) * 32 * ld
+    double* tmp = ring + (int64_t)(cmax + 1) * 32 * ld;            // 32 * ld
+    const int lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5;
+    const int rhs0 = warp * NR;
+    const double* F = fac + S.fac_off;
+    const int m = S.m;
+
+    double racc[MM][NR];
+#pragma unroll
+    for (int k = 0; k < MM; ++k)
+#pragma unroll
+        for (int j = 0; j < NR; ++j) racc[k][j] = 0.0;
+
+    // r' = r - alpha q for (system, rhs) pairs still iterating (see ResidIn)
+    double al[NR];
+    bool upd[NR];
+#pragma unroll
+    for (int j = 0; j < NR; ++j) {
+        al[j] = 0.0;
+        upd[j] = false;
+        if (qin != nullptr) {
+            const CgScalars cj = csc[(int64_t)S.seg * ld + rhs0 + j];
+            upd[j] = cj.active != 0;
+            if (upd[j]) al[j] = cj.alpha;
+        }
+    }
+    // Inputs of block row K (r and q rows, basis rows, row scale) are
+    // loaded two block rows ahead into alternating register buffers and
+    // kept in their loaded type until the step that uses them, so their
+    // global-memory latency overlaps the substitution of earlier rows.
+    auto load_fwd = [&](int K, double (&rv)[NR], double (&qv)[NR], double (&pv)[MM], double& scv) {
+        const int row = K * 32 + lane;
+        const bool valid = K < nb && row < n;
+        const int64_t grow = S.row0 + row;
+        scv = 1.0;
+#pragma unroll
+        for (int j = 0; j < NR; ++j) {
+            rv[j] = 0.0;
+            qv[j] = 0.0;
+        }
+#pragma unroll
+        for (int k = 0; k < MM; ++k) pv[k] = 0.0;
+        if (valid) {
+            if (rowscale != nullptr) scv = rowscale[grow];
+#pragma unroll
+            for (int j = 0; j < NR; ++j) {
+                rv[j] = rin[grow * ld + rhs0 + j];
+                if (upd[j]) qv[j] = qin[grow * ld + rhs0 + j];
+            }
+            if (rc != nullptr) {
+#pragma unroll
+                for (int k = 0; k < MM; ++k)
+                    if (k < m) pv[k] = psi[S.psi_off + (int64_t)row * m + k];
+            }
+        }
+    };
+    double rb[2][NR], qb[2][NR], sb[2];
+    double pb[2][MM];
+    load_fwd(0, rb[0], qb[0], pb[0], sb[0]);
+    load_fwd(1, rb[1], qb[1], pb[1], sb[1]);
+
+    // ---------------- forward ----------------
+    // one commit group per block row; row K+D is requested at step K
+    for (int j = 0; j < D; ++j) {
+        if (j < nb) block_copy_async(bufs + (int64_t)(j % nbuf) * brs_max, F + (int64_t)j * brs, brs * sizeof(double));
+        cp_async_commit();
+    }
+    auto fwd_step = [&](int K, double (&rv)[NR], double (&qv)[NR], double (&pb_)[MM], double& scv) {
+        if (K + D < nb)
+            block_copy_async(bufs + (int64_t)((K + D) % nbuf) * brs_max, F + (int64_t)(K + D) * brs,
+                             brs * sizeof(double));
+        cp_async_commit();
+        double t[NR], pv[MM];
+#pragma unroll
+        for (int j = 0; j < NR; ++j) t[j] = ((upd[j] ? fma(-al[j], qv[j], rv[j]) : rv[j]) * scv);
+#pragma unroll
+        for (int k = 0; k < MM; ++k) pv[k] = pb_[k];
+        load_fwd(K + 2, rv, qv, pb_, scv);
+        cp_async_wait_n(D);
+        __syncthreads();
+        const double* B = bufs + (int64_t)(K % nbuf) * brs_max;
+        const int row = K * 32 + lane;
+        const bool valid = row < n;
+        const int64_t grow = S.row0 + row;
+        if (rc != nullptr) {
+#pragma unroll
+            for (int k = 0; k < MM; ++k)
+#pragma unroll
+                for (int j = 0; j < NR; ++j) racc[k][j] += pv[k] * t[j];
+        }
+        for (int d = 0; d < c; ++d) {
+            const int src = K - c + d;
+            if (src < 0) continue;
+            const double* T = B + d * 1024;
+            const double* ys = ring + (int64_t)(src % (c + 1)) * 32 * ld + rhs0;
+#pragma unroll 8
+            for (int q = 0; q < 32; ++q) {
+                double coef = T[tile_idx(lane, q)];
+                if (d == 0 && q < lane) coef = 0.0;
+#pragma unroll
+                for (int j = 0; j < NR; ++j) t[j] -= coef * ys[q * ld + j];
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < NR; ++j) tmp[lane * ld + rhs0 + j] = t[j];
+        __syncwarp();
+        const double piv = B[c * 1024 + lane];
+        double y[NR];
+#pragma unroll
+        for (int j = 0; j < NR; ++j) y[j] = piv * t[j];
+#pragma unroll 8
+        for (int q = 0; q < 32; ++q) {
+            const double coef = q < lane ? B[tile_idx(lane, q)] : 0.0;
+#pragma unroll
+            for (int j = 0; j < NR; ++j) y[j] += coef * tmp[q * ld + rhs0 + j];
+        }
+        double* yr = ring + (int64_t)(K % (c + 1)) * 32 * ld + rhs0;
+#pragma unroll
+        for (int j = 0; j < NR; ++j) yr[lane * ld + j] = y[j];
+        if (valid) {
+#pragma unroll
+            for (int j = 0; j < NR; ++j) zf[grow * ld + rhs0 + j] = y[j];
+        }
+        __syncthreads();
+    };
+#pragma unroll 1
+    for (int K = 0; K < nb; K += 2) {
+        fwd_step(K, rb[0], qb[0], pb[0], sb[0]);
+        if (K + 1 < nb) fwd_step(K + 1, rb[1], qb[1], pb[1], sb[1]);
+    }
+    pdl_trigger();
+    // restriction: reduce over lanes, lane 0 writes r_c rows of this subdomain
+    if (rc != nullptr) {
+#pragma unroll
+        for (int k = 0; k < MM; ++k) {
+#pragma unroll
+            for (int j = 0; j < NR; ++j) {
+                double v = racc[k][j];
+                for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+                if (lane == 0 && k < m) rc[(S.coff + k) * ld + rhs0 + j] = v;
+            }
+        }
+    }
+    // ---------------- backward ----------------
+    // step K needs block rows K..K+c; row K-D is requested at step K
+    cp_async_wait_all();
+    __syncthreads();
+    for (int j = 0; j < D; ++j) {
+        const int r = nb - 1 - j;
+        if (r >= 0) block_copy_async(bufs + (int64_t)(r % nbuf) * brs_max, F + (int64_t)r * brs, brs * sizeof(double));
+        cp_async_commit();
+    }
+    auto load_bwd = [&](int K, double (&wv)[NR]) {
+        const int row = K * 32 + lane;
+        const bool valid = K >= 0 && row < n;
+        const int64_t grow = S.row0 + row;
+#pragma unroll
+        for (int j = 0; j < NR; ++j) wv[j] = 0.0;
+        if (valid) {
+#pragma unroll
+            for (int j = 0; j < NR; ++j) wv[j] = zf[grow * ld + rhs0 + j];
+        }
+    };
+    double wb[2][NR];
+    load_bwd(nb - 1, wb[0]);
+    load_bwd(nb - 2, wb[1]);
+    auto bwd_step = [&](int K, double (&wv)[NR]) {
+        if (K - D >= 0)
+            block_copy_async(bufs + (int64_t)((K - D) % nbuf) * brs_max, F + (int64_t)(K - D) * brs,
+                             brs * sizeof(double));
+        cp_async_commit();
+        double w[NR];
+#pragma unroll
+        for (int j = 0; j < NR; ++j) w[j] = wv[j];
+        load_bwd(K - 2, wv);
+        cp_async_wait_n(D);
+        __syncthreads();
+        const int row = K * 32 + lane;
+        const bool valid = row < n;
+        const int64_t grow = S.row0 + row;
+        for (int d = 1; d <= c; ++d) {
+            const int src = K + d;
+            if (src >= nb) break;
+            const double* Bs = bufs + (int64_t)(src % nbuf) * brs_max;
+            const double* T = (d < c) ? Bs + (c - d) * 1024 : Bs;
+            const double* xs = ring + (int64_t)(src % (c + 1)) * 32 * ld + rhs0;
+#pragma unroll 8
+            for (int r = 0; r < 32; ++r) {
+                double coef = T[tile_idx(r, lane)];
+                if (d == c && r > lane) coef = 0.0;
+#pragma unroll
+                for (int j = 0; j < NR; ++j) w[j] -= coef * xs[r * ld + j];
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < NR; ++j) tmp[lane * ld + rhs0 + j] = w[j];
+        __syncwarp();
+        const double* B = bufs + (int64_t)(K % nbuf) * brs_max;
+        const double piv = B[c * 1024 + lane];
+        double x[NR];
+#pragma unroll
+        for (int j = 0; j < NR; ++j) x[j] = piv * w[j];
+#pragma unroll 8
+        for (int r = 0; r < 32; ++r) {
+            const double coef = r > lane ? B[tile_idx(r, lane)] : 0.0;
+#pragma unroll
+            for (int j = 0; j < NR; ++j) x[j] += coef * tmp[r * ld + rhs0 + j];
+        }
+        double* xr = ring + (int64_t)(K % (c + 1)) * 32 * ld + rhs0;
+#pragma unroll
+        for (int j = 0; j < NR; ++j) xr[lane * ld + j] = x[j];
+        if (valid) {
+#pragma unroll
+            for (int j = 0; j < NR; ++j) zf[grow * ld + rhs0 + j] = x[j];
+        }
+        __syncthreads();
+    };
+#pragma unroll 1
+    for (int K = nb - 1; K >= 0; K -= 2) {
+        bwd_step(K, wb[0]);
+        if (K - 1 >= 0) bwd_step(K - 1, wb[1]);
+    }
+}
+
 // Shared memory that a setup or a launch shape is checked against: the
-// staging of c + depth + 1 block rows (an upper bound of what is used).
+// staging of c + depth + 1 block rows (what the lane-per-row kernel uses, an upper
+// bound for the other).
 size_t local_solve_smem(int cmax, int ld, size_t tf_bytes, int depth) {
     return ((size_t)(cmax + depth + 1) * blockrow_elems(cmax) + (size_t)(cmax + 1) * 32 * ld + 32 * ld) *
            tf_bytes;
@@ -349,8 +598,37 @@ static cudaError_t local_f64(const LocalSolveArgs& a, const double* fac, const d
                          a.in.sc, a.rowscale, zf, psi, rc, a.ld, a.ncols, a.cmax, depth, a.st);
 }
 
+template <int NR, int MM>
+static cudaError_t local_f64_rows(const LocalSolveArgs& a, const double* fac, const double* psi, double* zf, double* rc) {
+    int depth = a.depth > 0 ? a.depth : 4;
+    while (depth > 1 && local_solve_smem(a.cmax, a.ld, 8, depth) > (a.depth > 0 ? 200 : 100) * 1024) --depth;
+    const size_t smem = local_solve_smem(a.cmax, a.ld, 8, depth);
+    auto kern = k_local_f64_rows<NR, MM>;
+    static size_t smem_set = 0;           // per template instance
+    if (smem > smem_set) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        smem_set = smem;
+    }
+    return launch_kernel(a.pdl, kern, dim3(a.nsub), dim3(a.ld / NR * 32), smem, a.stream, a.subs, fac, a.in.r, a.in.q,
+                         a.in.sc, a.rowscale, zf, psi, rc, a.ld, a.cmax, depth, a.st);
+}
+
 template <int MM>
 static cudaError_t local_f64_mm(const LocalSolveArgs& a, const double* fac, const double* psi, double* zf, double* rc) {
+    // A lane per row where the FP64 pipe is full: one tile a block row and enough
+    // subdomains.  Lane per row / row pairs, us a launch at 1, 2, 3, 4 columns:
+    //   1024 subdomains of 32^2 (6.7 an SM)  293 / 730  512 / 860  967 / 1122  967 / 1304
+    //   361 of 16^2 (2.4)                     40 / 49   104 / 92   179 / 122   179 / 128
+    //   256 of 32^2 (1.7)                    247 / 238  430 / 288  758 / 387   758 / 402
+    //   1728 of 8^3 (11, two tiles)          395 / 379 1230 / 884 2156 / 1305 2156 / 1403
+    //   512 of 8^3 (3.4, two tiles)          199 / 131  597 / 298 1050 / 430  1050 / 461
+    constexpr int R4 = MM > 8 ? 2 : 4;   // columns a warp (registers)
+    if (a.cmax == 1 && a.ld <= 4 && a.nsub > (a.ld == 1 ? 2 : 4) * a.sms) {
+        if (a.ld == 1) return local_f64_rows<1, MM>(a, fac, psi, zf, rc);
+        if (a.ld == 2) return local_f64_rows<2, MM>(a, fac, psi, zf, rc);
+        return local_f64_rows<R4, MM>(a, fac, psi, zf, rc);
+    }
     if (a.ncols > 16) return local_f64<2, MM, 1>(a, fac, psi, zf, rc);
     // lanes per task: at least four warps, and no half-empty one where twice the lanes still fit a block
     int s = 1;

@@ -71,7 +71,8 @@ struct LocalSolveArgs {
     const SolveState* st;
     bool pdl;
     int depth;               // ring depth (block rows in flight); 0: default
-    int ncols;               // right-hand sides (<= ld); the columns beyond are left as they are
+    int ncols;               // right-hand sides (<= ld); the columns beyond may be left as they are
+    int sms;                 // SMs of the device
 };
 
 struct LocalTmaArgs {
