@@ -31,10 +31,12 @@
 // (bswz): head and tail of two consecutive rows of a column in 16
 // bytes, split once by the lane that made them.
 //
-// What bounds it: one row-major tile with scalar, separately addressed
-// fragment loads and cvt.rna splits issued about 12,000 warp instructions per block row at 32
-// right-hand sides where this one needs about 3,000; then the tensor pipe
-// (256 MMAs per block row and 16 columns) and the bytes of the factor.
+// What bounds it: row-major tiles with scalar, separately addressed fragment
+// loads and cvt.rna splits took 12,000 warp instructions a block row at 32
+// right-hand sides (both sweeps; issue 57 %, tensor pipe 18 %), this layout
+// 8,300 (8 columns a group; the tuned 16 take fewer).  What is left are fixed
+// latencies (a third of the stalls), shared memory, the tensor pipe (23 %) and the
+// bytes of the factor.
 //
 // Staging: one bulk copy per block row into a ring of depth + 1 slots with
 // bounded mbarrier waits.  The backward sweep is right-looking: x_K updates
