@@ -549,21 +549,32 @@ k_init_norms(const double* __restrict__ r, RedLayout R, CgScalars* sc, SolveStat
 }
 
 // Caller order (column-major n x nrhs) <-> internal node-major rows, through a
-// shared-memory tile of 2048 values: both sides move whole lines (a column of
-// consecutive dofs, a row's LD values), where a thread per dof wrote or read 8
-// bytes of a different row per lane.  Bound by HBM (apply and
-// product at 96^3 x 16, two permutes in and two out: 1.00 -> 0.85 ms).
-constexpr int kPermTile = 2048;
+// shared-memory tile of at most 256 rows and 2048 values: both sides move whole
+// lines (a column of consecutive dofs, a row's LD values), where a thread per
+// dof wrote or read 8 bytes of a different row per lane.  Bound by HBM (apply and
+// product at 96^3 x 16, two permutes in and two out: 1.00 -> 0.85 ms).  One column
+// has whole lines on both sides as it is and needs no tile: a row's index and
+// its value load together, and 256 rows a block fill more SMs than 2048.
+__host__ __device__ constexpr int perm_rows(int ld) { return ld < 8 ? 256 : 2048 / ld; }
 template <int LD>
 __global__ void __launch_bounds__(256)
 k_permute_in(const double* __restrict__ f, int64_t n, int nrhs, const int64_t* __restrict__ int_row,
              double* __restrict__ r, double* __restrict__ x) {
-    constexpr int ROWS = kPermTile / LD;
+    constexpr int ROWS = perm_rows(LD);
+    if constexpr (LD == 1) {
+        const int64_t i = (int64_t)blockIdx.x * ROWS + threadIdx.x;
+        if (i >= n) return;
+        const int64_t row = __ldg(int_row + i);
+        if (!AMS_ROW_OK(row, 6)) return;
+        r[row] = f[i];
+        if (x != nullptr) x[row] = 0.0;
+        return;
+    }
     __shared__ double tile[ROWS * (LD + 1)];
     const int64_t i0 = (int64_t)blockIdx.x * ROWS;
     const int nr = (int)(n - i0 < ROWS ? n - i0 : ROWS);
 #pragma unroll 4
-    for (int e = threadIdx.x; e < kPermTile; e += 256) {
+    for (int e = threadIdx.x; e < ROWS * LD; e += 256) {
         const int i = e % ROWS, k = e / ROWS;
         tile[i * (LD + 1) + k] = i < nr && k < nrhs ? f[i0 + i + (int64_t)k * n] : 0.0;
     }
@@ -582,7 +593,14 @@ template <int LD, typename XT>
 __global__ void __launch_bounds__(256)
 k_permute_out(const XT* __restrict__ x, int64_t n, int nrhs, const int64_t* __restrict__ int_row,
               double* __restrict__ u) {
-    constexpr int ROWS = kPermTile / LD;
+    constexpr int ROWS = perm_rows(LD);
+    if constexpr (LD == 1) {
+        const int64_t i = (int64_t)blockIdx.x * ROWS + threadIdx.x;
+        if (i >= n) return;
+        const int64_t row = __ldg(int_row + i);
+        u[i] = AMS_ROW_OK(row, 6) ? widen(x[row]) : 0.0;
+        return;
+    }
     __shared__ XT tile[ROWS * (LD + 1)];
     const int64_t i0 = (int64_t)blockIdx.x * ROWS;
     const int nr = (int)(n - i0 < ROWS ? n - i0 : ROWS);
@@ -747,7 +765,7 @@ void launch_prolong_update(const LaunchCtx& L, int prec, const ProlongArgs& a) {
     else prolong_tp<float, __nv_bfloat16>(L, a);
 }
 
-static unsigned perm_blocks(int64_t n, int ld) { return (unsigned)((n * ld + kPermTile - 1) / kPermTile); }
+static unsigned perm_blocks(int64_t n, int ld) { return (unsigned)((n + perm_rows(ld) - 1) / perm_rows(ld)); }
 template <int LD>
 static void perm_in_ld(cudaStream_t s, const double* f, int64_t n, int nrhs, const int64_t* int_row, double* r, double* x) {
     k_permute_in<LD><<<perm_blocks(n, LD), 256, 0, s>>>(f, n, nrhs, int_row, r, x);
