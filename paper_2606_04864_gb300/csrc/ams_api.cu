@@ -1476,7 +1476,7 @@ static ams_status estimate_two_grid_omega(ams_handle h) {
 // the prolongation (each subdomain multiplies its rows of the backward block
 // with y); with more, the per-subdomain gathers of y cost more than the
 // separate backward launch.
-static bool fused_backward(int ld) { return ld <= 4; }
+static bool fused_backward(int ld) { return ld <= kFusedBackwardMaxLd; }
 
 // forward coarse substitution y = L_c^{-1} r_c, and the backward one when it
 // is not fused
@@ -1496,7 +1496,7 @@ static int launch_coarse(ams_handle h, int ld, bool with_state) {
 // of p less per iteration; measured faster at 32 right-hand sides).  With
 // fewer the prolongation is latency-bound and gains nothing from the bytes,
 // while the direction update would pay for them: the update stays there.
-static bool defer_x_update(int ld) { return ld >= 8; }
+static bool defer_x_update(int ld) { return ld >= kDeferXMinLd; }
 
 static ProlongArgs prolong_args(ams_handle h, int mode, const double* p, int ld) {
     const bool coarse = h->Nc > 0, fused = fused_backward(ld);
@@ -1534,7 +1534,7 @@ static ams_status apply_two_grid(ams_handle h, const LaunchCtx& L, int mode, con
         prof_end(h);
     }
     prof_begin(h, AMS_KERNEL_PROLONG);
-    launch_prolong_update(L2, h->prec, prolong_args(h, 0, p, L.ld));   // z = x^2
+    AMS_CUDA_TRY(launch_prolong_update(L2, h->prec, prolong_args(h, 0, p, L.ld)));   // z = x^2
     launch_tg_resid(L2, h->d_z, h->prec == AMS_PREC_FP64, rin, h->d_tw);   // z in the apply precision
     prof_end(h);
     prof_begin(h, AMS_KERNEL_LOCAL);
@@ -1546,7 +1546,7 @@ static ams_status apply_two_grid(ams_handle h, const LaunchCtx& L, int mode, con
     a.yc = nullptr;
     a.qmat = nullptr;
     prof_begin(h, AMS_KERNEL_PROLONG);
-    launch_prolong_update(L2, h->prec, a);
+    AMS_CUDA_TRY(launch_prolong_update(L2, h->prec, a));
     prof_end(h);
     h->launches += 5 + local_extra_launches(h, L.ld);   // prolongation, residual, local solves, combine, prolongation
     AMS_CUDA_TRY(cudaGetLastError());
@@ -1574,7 +1574,7 @@ static ams_status apply_precond(ams_handle h, const LaunchCtx& L, int mode, cons
     LaunchCtx L2 = L;
     if (!with_state) L2.st = nullptr;
     prof_begin(h, AMS_KERNEL_PROLONG);
-    launch_prolong_update(L2, h->prec, prolong_args(h, mode, p, L.ld));
+    AMS_CUDA_TRY(launch_prolong_update(L2, h->prec, prolong_args(h, mode, p, L.ld)));
     prof_end(h);
     AMS_CUDA_TRY(cudaGetLastError());
     return AMS_OK;
@@ -1852,7 +1852,7 @@ static ams_status autotune(ams_handle h, const double* f_dev, int nrhs, int ld) 
             AMS_TRY(ctx(&L));
             float ms = 0.f;
             AMS_TRY(timed_after([]() -> ams_status { return AMS_OK; }, [&]() -> ams_status {
-                launch_prolong_update(L, h->prec, prolong_args(h, 2, h->d_p2, ld));
+                AMS_CUDA_TRY(launch_prolong_update(L, h->prec, prolong_args(h, 2, h->d_p2, ld)));
                 return AMS_OK;
             }, &ms));
             if (ms < best) {
@@ -2501,7 +2501,9 @@ ams_status ams_time_kernel(ams_handle h, int32_t which, int32_t reps, double* av
                 AMS_TRY(launch_local(h, ld, ResidIn{h->d_r, h->d_q, h->d_sc}, true));
                 break;
             case AMS_KERNEL_COARSE: launch_coarse(h, ld, true); break;
-            case AMS_KERNEL_PROLONG: launch_prolong_update(L, h->prec, prolong_args(h, 2, h->d_p2, ld)); break;
+            case AMS_KERNEL_PROLONG:
+                AMS_CUDA_TRY(launch_prolong_update(L, h->prec, prolong_args(h, 2, h->d_p2, ld)));
+                break;
         }
         return AMS_OK;
     };

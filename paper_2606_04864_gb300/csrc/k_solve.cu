@@ -253,7 +253,8 @@ k_prolong_update(const SubInfo* __restrict__ subs, const TP* __restrict__ psi, c
                  const TF* __restrict__ zf, double* __restrict__ r, const double* __restrict__ q,
                  double* __restrict__ x, const double* __restrict__ p, TF* __restrict__ z, RedLayout R,
                  CgScalars* sc, SolveState* st, int nseg, const int32_t* __restrict__ sub_of_row) {
-    constexpr bool ITER = MODE >= 2, FLEX = MODE == 3, XUPD = ITER && LD < 8;
+    constexpr bool ITER = MODE >= 2, FLEX = MODE == 3, XUPD = ITER && LD < kDeferXMinLd;
+    constexpr bool FUSED = LD <= kFusedBackwardMaxLd;   // has the code and the scratch for qmat
     using AT = typename Acc<TF>::type;
     using V4 = typename std::conditional<sizeof(TF) == 4, float4, double4>::type;
     constexpr int NCG = kRedThreads / LD;            // column groups of the backward product
@@ -265,7 +266,7 @@ k_prolong_update(const SubInfo* __restrict__ subs, const TP* __restrict__ psi, c
     constexpr int kChunk = !CH ? 1 : CH0 > 16 ? 16 : CH0;
     static_assert(kChunk >= 1, "one block of e_c fits");
     __shared__ AT s_ec[kChunk * MM * LD];
-    __shared__ AT s_part[LD < 8 ? NW * MM * LD : 1];
+    __shared__ AT s_part[FUSED ? NW * MM * LD : 1];
     __shared__ int64_t s_psi[kChunk];                // basis offset of the subdomain's row 0, less row0 * m
     __shared__ int s_mv[kChunk];                     // modes, and how its basis rows load
     pdl_wait();
@@ -368,50 +369,52 @@ k_prolong_update(const SubInfo* __restrict__ subs, const TP* __restrict__ psi, c
         for (int64_t si = s_lo; si < s_hi; ++si) {
             const SubInfo S = subs[si];
             const int m = S.m;
-            const bool coarse = (ec != nullptr || qmat != nullptr) && m > 0;
+            const bool coarse = (ec != nullptr || (FUSED && qmat != nullptr)) && m > 0;
             if (coarse && ec != nullptr) {
                 // e_c computed by a separate backward-substitution launch
                 for (int i = threadIdx.x; i < MM * LD; i += kRedThreads)
                     s_ec[i] = (i < m * LD) ? (AT)ec[(int64_t)S.coff * LD + i] : AT(0);
             } else if (coarse) {
-                // e_c rows of this subdomain: acc[k] = sum_j Q[k][j] y[gat[j]] over this thread's columns
-                const CoarseRef cr = cref[si];
-                const TF* Q = qmat + cr.q_off;
-                const int32_t* G = gat + cr.gat_off;
-                AT acc[MM];
+                if constexpr (FUSED) {
+                    // e_c rows of this subdomain: acc[k] = sum_j Q[k][j] y[gat[j]] over this thread's columns
+                    const CoarseRef cr = cref[si];
+                    const TF* Q = qmat + cr.q_off;
+                    const int32_t* G = gat + cr.gat_off;
+                    AT acc[MM];
 #pragma unroll
-                for (int k = 0; k < MM; ++k) acc[k] = AT(0);
-                for (int c4 = cg; 4 * c4 < cr.K; c4 += NCG) {
-                    const int j0 = 4 * c4;
-                    AT yv[4];
+                    for (int k = 0; k < MM; ++k) acc[k] = AT(0);
+                    for (int c4 = cg; 4 * c4 < cr.K; c4 += NCG) {
+                        const int j0 = 4 * c4;
+                        AT yv[4];
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        yv[e] = AT(0);
-                        if (j0 + e < cr.K) {
-                            const int gi = __ldg(G + j0 + e);
-                            if (AMS_COARSE_OK(gi, 2)) yv[e] = (AT)yc[(int64_t)gi * LD + rhs];
+                        for (int e = 0; e < 4; ++e) {
+                            yv[e] = AT(0);
+                            if (j0 + e < cr.K) {
+                                const int gi = __ldg(G + j0 + e);
+                                if (AMS_COARSE_OK(gi, 2)) yv[e] = (AT)yc[(int64_t)gi * LD + rhs];
+                            }
+                        }
+#pragma unroll
+                        for (int k = 0; k < MM; ++k) {
+                            if (k < m) {
+                                const V4 qv = *reinterpret_cast<const V4*>(Q + (int64_t)k * cr.ldm + j0);
+                                acc[k] += (AT)qv.x * yv[0] + (AT)qv.y * yv[1] + (AT)qv.z * yv[2] + (AT)qv.w * yv[3];
+                            }
                         }
                     }
+                    // sum over column groups: lanes of a warp with the same rhs, then warps in order
 #pragma unroll
                     for (int k = 0; k < MM; ++k) {
-                        if (k < m) {
-                            const V4 qv = *reinterpret_cast<const V4*>(Q + (int64_t)k * cr.ldm + j0);
-                            acc[k] += (AT)qv.x * yv[0] + (AT)qv.y * yv[1] + (AT)qv.z * yv[2] + (AT)qv.w * yv[3];
-                        }
+                        AT a = acc[k];
+                        for (int off = 16; off >= LD; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+                        if (lane < LD) s_part[(warp * MM + k) * LD + lane] = a;
                     }
-                }
-                // sum over column groups: lanes of a warp with the same rhs, then warps in order
-#pragma unroll
-                for (int k = 0; k < MM; ++k) {
-                    AT a = acc[k];
-                    for (int off = 16; off >= LD; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
-                    if (lane < LD) s_part[(warp * MM + k) * LD + lane] = a;
-                }
-                __syncthreads();
-                for (int i = threadIdx.x; i < MM * LD; i += kRedThreads) {
-                    AT a = AT(0);
-                    for (int w = 0; w < NW; ++w) a += s_part[w * MM * LD + i];
-                    s_ec[i] = a;
+                    __syncthreads();
+                    for (int i = threadIdx.x; i < MM * LD; i += kRedThreads) {
+                        AT a = AT(0);
+                        for (int w = 0; w < NW; ++w) a += s_part[w * MM * LD + i];
+                        s_ec[i] = a;
+                    }
                 }
             }
             __syncthreads();
@@ -720,15 +723,14 @@ void launch_init_norms(const LaunchCtx& L, const double* r, int nrhs) {
 }
 
 template <typename TF, typename TP, int LD, int MM, bool CH>
-static void prolong_ch(const LaunchCtx& L, const ProlongArgs& a) {
+static cudaError_t prolong_ch(const LaunchCtx& L, const ProlongArgs& a) {
     auto kern = a.mode == 0   ? k_prolong_update<TF, TP, LD, MM, 0, CH>
                 : a.mode == 1 ? k_prolong_update<TF, TP, LD, MM, 1, CH>
                 : a.flexible  ? k_prolong_update<TF, TP, LD, MM, 3, CH>
                               : k_prolong_update<TF, TP, LD, MM, 2, CH>;
-    launch_kernel(L.pdl, kern, dim3((unsigned)L.nblk_sub), dim3(kRedThreads), 0, L.stream, L.subs, (const TP*)a.psi,
-                  (const TF*)a.ec, (const TF*)a.yc, (const TF*)a.qmat, a.cref, a.gat, (const TF*)a.zf, a.r, a.q, a.x, a.p,
-                  (TF*)a.z,
-                  L.red_sub, L.sc, L.st, L.nseg, L.sub_of_row);
+    return launch_kernel(L.pdl, kern, dim3((unsigned)L.nblk_sub), dim3(kRedThreads), 0, L.stream, L.subs,
+                         (const TP*)a.psi, (const TF*)a.ec, (const TF*)a.yc, (const TF*)a.qmat, a.cref, a.gat,
+                         (const TF*)a.zf, a.r, a.q, a.x, a.p, (TF*)a.z, L.red_sub, L.sc, L.st, L.nseg, L.sub_of_row);
 }
 // In chunks up to 2048 elements a subdomain on average, two passes of a block
 // over it.  One subdomain at a time / in chunks, us a launch: 1430 elements (the
@@ -736,33 +738,34 @@ static void prolong_ch(const LaunchCtx& L, const ProlongArgs& a) {
 // (77^3 x 8) 84 / 86, 4096 (64^3 x 8) 53 / 55, 8192 (96^3 x 16) 200 / 204, where
 // the row's subdomain is one more load before the basis.  FP64 62 / 65 at 2900.
 template <typename TF, typename TP, int LD, int MM>
-static void prolong_mm(const LaunchCtx& L, const ProlongArgs& a) {
+static cudaError_t prolong_mm(const LaunchCtx& L, const ProlongArgs& a) {
     if constexpr (LD >= 8 && sizeof(TF) == 4) {
         if (L.rows * LD <= 2048 * (int64_t)L.nsub) return prolong_ch<TF, TP, LD, MM, true>(L, a);
     }
-    prolong_ch<TF, TP, LD, MM, false>(L, a);
+    return prolong_ch<TF, TP, LD, MM, false>(L, a);
 }
 template <typename TF, typename TP, int LD>
-static void prolong_ld(const LaunchCtx& L, const ProlongArgs& a) {
-    if (L.nsub == 0) return;
-    if (a.mmax > 8) prolong_mm<TF, TP, LD, kMaxM>(L, a);
-    else prolong_mm<TF, TP, LD, 8>(L, a);
+static cudaError_t prolong_ld(const LaunchCtx& L, const ProlongArgs& a) {
+    if (L.nsub == 0) return cudaSuccess;
+    return a.mmax > 8 ? prolong_mm<TF, TP, LD, kMaxM>(L, a) : prolong_mm<TF, TP, LD, 8>(L, a);
 }
 template <typename TF, typename TP>
-static void prolong_tp(const LaunchCtx& L, const ProlongArgs& a) {
+static cudaError_t prolong_tp(const LaunchCtx& L, const ProlongArgs& a) {
     switch (L.ld) {
-        case 1: prolong_ld<TF, TP, 1>(L, a); break;
-        case 2: prolong_ld<TF, TP, 2>(L, a); break;
-        case 4: prolong_ld<TF, TP, 4>(L, a); break;
-        case 8: prolong_ld<TF, TP, 8>(L, a); break;
-        case 16: prolong_ld<TF, TP, 16>(L, a); break;
-        default: prolong_ld<TF, TP, 32>(L, a); break;
+        case 1: return prolong_ld<TF, TP, 1>(L, a);
+        case 2: return prolong_ld<TF, TP, 2>(L, a);
+        case 4: return prolong_ld<TF, TP, 4>(L, a);
+        case 8: return prolong_ld<TF, TP, 8>(L, a);
+        case 16: return prolong_ld<TF, TP, 16>(L, a);
+        default: return prolong_ld<TF, TP, 32>(L, a);
     }
 }
-void launch_prolong_update(const LaunchCtx& L, int prec, const ProlongArgs& a) {
-    if (prec == AMS_PREC_FP64) prolong_tp<double, double>(L, a);
-    else if (prec == AMS_PREC_FP32) prolong_tp<float, float>(L, a);
-    else prolong_tp<float, __nv_bfloat16>(L, a);
+cudaError_t launch_prolong_update(const LaunchCtx& L, int prec, const ProlongArgs& a) {
+    if (a.qmat != nullptr && L.ld > kFusedBackwardMaxLd) return cudaErrorInvalidValue;
+    if (a.x == nullptr && a.mode == 2 && L.ld < kDeferXMinLd) return cudaErrorInvalidValue;
+    if (prec == AMS_PREC_FP64) return prolong_tp<double, double>(L, a);
+    if (prec == AMS_PREC_FP32) return prolong_tp<float, float>(L, a);
+    return prolong_tp<float, __nv_bfloat16>(L, a);
 }
 
 static unsigned perm_blocks(int64_t n, int ld) { return (unsigned)((n + perm_rows(ld) - 1) / perm_rows(ld)); }

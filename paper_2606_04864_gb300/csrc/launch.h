@@ -151,6 +151,12 @@ cudaError_t make_tile_map(void* base, int64_t rows, struct CUtensorMap_st* out);
 void launch_band_pack_tiles(cudaStream_t s, int nwork, const SubInfo* subs, const int64_t* band_off,
                             const int2* work, const double* band, const int64_t* out_off, float* fwd, float* mma,
                             float* piv);
+// Right-hand-side strides up to which the prolongation itself multiplies its
+// rows of the backward coarse block (ProlongArgs::qmat), and from which
+// x += alpha p rides on the next direction update instead of on it.  The host
+// chooses the arguments by these, the kernel compiles only what they let through.
+constexpr int kFusedBackwardMaxLd = 4;
+constexpr int kDeferXMinLd = 8;
 struct ProlongArgs {
     const void* psi;
     const void* ec;          // coarse correction from a separate backward launch, or NULL
@@ -168,7 +174,8 @@ struct ProlongArgs {
     int flexible;
     int mode;                // 0 apply only, 1 first application, 2 CG iteration
 };
-void launch_prolong_update(const LaunchCtx& L, int prec, const ProlongArgs& a);
+// cudaErrorInvalidValue, and no launch, for arguments that this stride's kernel has no code for.
+cudaError_t launch_prolong_update(const LaunchCtx& L, int prec, const ProlongArgs& a);
 
 // multiplicative two-grid cycle (k_two_grid.cu); v_is_fp64: v holds doubles,
 // else the apply precision's floats
