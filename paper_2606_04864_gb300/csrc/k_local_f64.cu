@@ -39,8 +39,10 @@ __device__ __forceinline__ double lane_sum(double v) {
 // NT tasks per thread (1: up to 16 right-hand sides, 2: up to 32); S lanes
 // per task, each taking every S-th term of its dot products.  A warp's
 // multiply-adds run on its own quarter of the SM at a quarter of the rate, so
-// S fills the last warp and gives a block at least four.
-template <int NT, int MM, int S>
+// S fills the last warp and gives a block at least four.  PAD: there are
+// columns between the right-hand sides and ld; they have no task, but the
+// coarse products and the prolongation read them, so they get zeros.
+template <int NT, int MM, int S, bool PAD>
 __global__ void __launch_bounds__(256)
 k_local_f64(const SubInfo* __restrict__ subs, const double* __restrict__ fac, const double* __restrict__ rin,
             const double* __restrict__ qin, const CgScalars* __restrict__ csc, const double* __restrict__ rowscale,
@@ -319,6 +321,14 @@ k_local_f64(const SubInfo* __restrict__ subs, const double* __restrict__ fac, co
         }
         cp_async_wait_n(D - 1);                // block row K - 1 has landed (the next barrier shows it to all)
     }
+    if constexpr (PAD) {
+        const int npad = ld - ncols;
+        for (int i = threadIdx.x; i < n * npad; i += blockDim.x)
+            zf[(sub.row0 + i / npad) * ld + ncols + i % npad] = 0.0;
+        if (rc != nullptr)
+            for (int i = threadIdx.x; i < m * npad; i += blockDim.x)
+                rc[(sub.coff + i / npad) * ld + ncols + i % npad] = 0.0;
+    }
 }
 
 // One to four right-hand sides on many subdomains of one tile a block row: a
@@ -580,13 +590,13 @@ static size_t local_f64_smem(int cmax, int ncols, int depth) {
     return ((size_t)(depth + 1) * blockrow_elems(cmax) + (size_t)(2 * cmax + 1) * 32 * ncols) * sizeof(double);
 }
 
-template <int NT, int MM, int S>
-static cudaError_t local_f64(const LocalSolveArgs& a, const double* fac, const double* psi, double* zf, double* rc) {
+template <int NT, int MM, int S, bool PAD>
+static cudaError_t local_f64_pad(const LocalSolveArgs& a, const double* fac, const double* psi, double* zf, double* rc) {
     // two block rows in flight hide the copies behind the FP64 pipe, and leave room for several blocks
     int depth = a.depth > 0 ? a.depth : 2;
     while (depth > 1 && local_f64_smem(a.cmax, a.ncols, depth) > 200 * 1024) --depth;
     const size_t smem = local_f64_smem(a.cmax, a.ncols, depth);
-    auto kern = k_local_f64<NT, MM, S>;
+    auto kern = k_local_f64<NT, MM, S, PAD>;
     static size_t smem_set = 0;           // per template instance
     if (smem > smem_set) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -596,6 +606,12 @@ static cudaError_t local_f64(const LocalSolveArgs& a, const double* fac, const d
     const int threads = ((16 * a.ncols * S / NT + 31) / 32) * 32;
     return launch_kernel(a.pdl, kern, dim3(a.nsub), dim3(threads), smem, a.stream, a.subs, fac, a.in.r, a.in.q,
                          a.in.sc, a.rowscale, zf, psi, rc, a.ld, a.ncols, a.cmax, depth, a.st);
+}
+
+template <int NT, int MM, int S>
+static cudaError_t local_f64(const LocalSolveArgs& a, const double* fac, const double* psi, double* zf, double* rc) {
+    return a.ncols < a.ld ? local_f64_pad<NT, MM, S, true>(a, fac, psi, zf, rc)
+                          : local_f64_pad<NT, MM, S, false>(a, fac, psi, zf, rc);
 }
 
 template <int NR, int MM>

@@ -71,7 +71,7 @@ struct LocalSolveArgs {
     const SolveState* st;
     bool pdl;
     int depth;               // ring depth (block rows in flight); 0: default
-    int ncols;               // right-hand sides (<= ld); the columns beyond may be left as they are
+    int ncols;               // right-hand sides (<= ld); zf and rc get zeros in the columns beyond
     int sms;                 // SMs of the device
 };
 
