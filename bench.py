@@ -51,7 +51,7 @@ METRIC = "PCG time-to-solution at rtol 1e-8 (s), iters, HBM GB/s; mixed vs FP64"
 WORKLOADS = ("grf3d_128_rhs32", "channels2d_1024", "grf3d_96", "batch48_uneven")
 
 # Kernel behind each timed solve slot, for the ncu traffic lookup.
-SLOT_KERNELS = {"local_solve_restrict": ("k_local_mma", "k_local_tma1"),
+SLOT_KERNELS = {"local_solve_restrict": ("k_local_mma", "k_local_tma1", "k_local_few"),
                 "spmv_direction": ("k_spmv_dot",),
                 "coarse_solve": ("k_coarse_mma", "k_coarse_gemm", "k_coarse_rows"),
                 "prolong_update": ("k_prolong_update",)}

@@ -79,8 +79,8 @@ typedef struct {
                                     number of right-hand sides, time candidate
                                     launch shapes (blocks per SM of the SpMV and
                                     prolongation grids, local-solve ring depth,
-                                    right-hand sides per warp of the several-RHS
-                                    local solve, L2 priorities of the one-RHS
+                                    how the local solve splits its right-hand
+                                    sides over warps, L2 priorities of the one-RHS
                                     local solve's tile copies) on that right-hand
                                     side and keep the fastest */
     int32_t coarse;              /* 1: two-level (default); 0: local solves only */
@@ -346,10 +346,10 @@ ams_status ams_get_info(ams_handle h, ams_info* info);
  * (1 <= nrhs <= 32; shapes are kept per nrhs rounded up to a power of two).
  * shape[0]  blocks per SM of the element-layout grids (direction update, SpMV)
  * shape[1]  blocks per SM of the subdomain-layout grid (prolongation)
- * shape[2]  local-solve ring depth in band tiles; 0 = derived from the band width
- * shape[3]  right-hand sides per warp of the several-RHS local solve (2, 4 or 8
- *           below 8 right-hand sides; 8 or 16 from 8 on, where the tile
- *           products run on the tensor cores); 0 = default
+ * shape[2]  local-solve ring depth in block rows; 0 = derived from the band width
+ * shape[3]  how the several-RHS local solve splits its right-hand sides: up to
+ *           four, 2 or 4 per warp; from five on, where the tile products run
+ *           on the tensor cores, 8 or (from 16) 16 per two warps; 0 = default
  * shape[4]  L2 priorities of the one-RHS local solve's factor-tile copies:
  *           0 none (default); 1 evict-first on copies that read a block row
  *           for the last time; 2 as 1, plus evict-last on the kept copies
@@ -363,9 +363,8 @@ ams_status ams_get_info(ams_handle h, ams_info* info);
  * and drops the iteration graph captured with the previous shapes; call it
  * between solves.  Errors: AMS_ERR_INVALID_ARG (NULL, nrhs out of range,
  * blocks per SM outside 1..8, depth outside 0..6, below 2 with TMA staging or
- * needing more than 200 KB of shared memory, right-hand sides per warp not
- * 0 or one of the values above, above the rounded count or leaving more
- * than 8 warps per block (4 from 8 right-hand sides on),
+ * needing more than 200 KB of shared memory, a split that is not 0 or one of
+ * the values above or is above the rounded count,
  * L2 mode outside 0..2, negative kept rows).
  */
 ams_status ams_get_launch_shape(ams_handle h, int32_t nrhs, int32_t* shape);

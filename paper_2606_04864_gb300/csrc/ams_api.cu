@@ -72,7 +72,7 @@ struct TuneCfg {
     int bps_elem = kRedBlocksPerSM;     // element-layout blocks per SM (direction update, SpMV)
     int bps_sub = kRedBlocksPerSM;      // subdomain-layout blocks per SM (prolongation)
     int depth = 0;                      // local-solve ring depth; 0: chosen from the band width
-    int nr = 0;                         // several-RHS local solve: right-hand sides per warp; 0: default
+    int nr = 0;                         // several-RHS local solve: right-hand sides per warp or warp pair; 0: default
     int l2mode = 0;                     // one-RHS local solve: L2 priorities of the factor tiles (0 none)
     int l2keep = 0;                     // block rows whose forward load keeps its L2 priority
     bool done = false;                  // autotuned
@@ -121,8 +121,8 @@ struct ams_handle_s {
     int32_t N = 0;
     int64_t Nc = 0;
     int cmax = 1, mmax = 0, nbmax = 1;
-    // subdomains grouped by band width (several-RHS local solve: one launch
-    // per group; empty when every subdomain has the same width)
+    // subdomains grouped by band width (all local solves but the one-vector
+    // one: a launch per group; empty when every subdomain has the same width)
     std::vector<int> cls_c, cls_n, cls_nb;
     int32_t* d_cls_order = nullptr;
     int num_sms = 1;                    // SMs of the handle's device
@@ -1366,10 +1366,11 @@ static LocalTmaArgs local_tma_args(ams_handle h, int ld, const ResidIn& in, bool
     return a;
 }
 
-// Launches of one local-solve pass beyond the first: the several-RHS
-// kernel launches once per band-width group.
+// Launches of one local-solve pass beyond the first: all but the one-vector
+// kernel launch once per band-width group.
 static int local_extra_launches(ams_handle h, int ld) {
-    return (h->use_tma && ld >= 2 && h->cls_c.size() > 1) ? (int)h->cls_c.size() - 1 : 0;
+    if (!h->use_tma || h->cls_c.size() <= 1 || local_one_vector(local_tma_args(h, ld, ResidIn{}, false))) return 0;
+    return (int)h->cls_c.size() - 1;
 }
 
 static ams_status launch_local(ams_handle h, int ld, const ResidIn& in, bool with_state,
@@ -1803,11 +1804,12 @@ static ams_status autotune(ams_handle h, const double* f_dev, int nrhs, int ld) 
         // the right depth depends on the group's size.  The right-looking kernels (all but the one-RHS
         // one) gain nothing from more than a few rows in flight and lose occupancy to them.
         const ResidIn in{h->d_r, h->d_q, h->d_sc};
-        const bool one_rhs = h->use_tma && ld == 1, groups = h->use_tma && ld >= 16;
+        const bool one_rhs = h->use_tma && ld == 1;
+        const int nr_hi = !h->use_tma ? 0 : ld >= 16 ? 16 : ld == 4 ? 4 : 0, nr_lo = nr_hi / 2;   // 0: no choice
         const int dmin = h->use_tma ? 2 : 1, dmax = one_rhs ? 6 : h->use_tma ? 4 : 3;
         float best = 1e30f;
         int arg = 0, argn = 0;
-        for (int nr = groups ? 16 : 0; nr == 0 || nr >= 8; nr = nr == 0 ? 1 : nr / 2) {
+        for (int nr = nr_hi; nr >= nr_lo; nr = nr > nr_lo ? nr_lo : -1) {
             for (int d = dmin; d <= dmax; ++d) {
                 const size_t smem = h->use_tma ? local_tma_launch_smem(local_tma_args(h, ld, in, true), d)
                                                : local_solve_smem(h->cmax, ld, h->tf_bytes(), d);
@@ -2278,11 +2280,11 @@ ams_status ams_set_launch_shape(ams_handle h, int32_t nrhs, const int32_t* shape
             return AMS_ERR_INVALID_ARG;
         }
     }
-    const bool nr_ok = ld >= 8 ? ((nr == 8 || nr == 16) && nr <= ld && ld / nr <= 4)
-                               : ((nr == 2 || nr == 4 || nr == 8) && nr <= ld && ld / nr <= 8);
+    const bool nr_ok = ld >= 8 ? (nr == 8 || nr == 16) && nr <= ld
+                               : (nr == 2 || nr == 4) && nr <= ld;
     if (nr != 0 && !nr_ok) {
-        set_error("right-hand sides per warp must be 0, or (below 8 right-hand sides) 2, 4 or 8 with at most "
-                  "8 warps per block, or (8 or more) 8 or 16 with at most 4 warps per block");
+        set_error("right-hand sides per warp must be 0, or 2 or 4 (up to four right-hand sides) or 8 or 16 (from five, "
+                  "per two warps), and no more than the count rounded up to a power of two");
         return AMS_ERR_INVALID_ARG;
     }
     if (l2mode < 0 || l2mode > 2 || l2keep < 0) {

@@ -1,4 +1,4 @@
-// Local solves for several right-hand sides on the tensor cores (Section 3.2:
+// Local solves for five and more right-hand sides on the tensor cores (Section 3.2:
 // z_f = sum_i R_i^T A_i^{-1} R_i r' with A_i = L_i L_i^T, and the restriction
 // r_c = R_0 r' of the coarse correction, Section 3.1, fused in).
 //
@@ -9,8 +9,9 @@
 // and a tail and the product is summed as tail*head + head*tail + head*head,
 // which keeps the apply at FP32 accuracy (the dropped tail*tail term is below
 // FP32 rounding); BF16 basis entries are exact in TF32 and are not split.
-// Two to seven right-hand sides (and one, on subdomains too large for the
-// one-vector kernel) use the same kernel with empty columns.
+// Five to seven right-hand sides have a stride of 8 like eight.  Up to four, all
+// in FP32 multiply-adds, are k_local_few's (k_local_tma.cu), which is faster
+// there and closer to the FP64 apply.
 //
 // Why warp-level MMAs rather than tcgen05: one subdomain's solve is a
 // chain of dependent 32-row steps, and tcgen05.mma needs M >= 64 rows per
@@ -50,8 +51,7 @@
 //
 // Measured (us a launch, row-major kernel with one warp per 8 columns before):
 // 128^3 x 32 1224 -> 711-750, 96^3 x 16 314 -> 183, 8 uneven systems x 8
-// 406 -> 172, 77^3 x 8 (cycle, with its scaling) 222 -> 105, 96x80x72 x 3
-// 152 -> 117, 64^3 x 8 91 -> 57.  One warp per column group with both row
+// 406 -> 172, 77^3 x 8 (cycle, with its scaling) 222 -> 105, 64^3 x 8 91 -> 57.  One warp per column group with both row
 // halves: 32: 742, 16: 191, 8 uneven systems 192, 64^3 x 8 68.
 #include <algorithm>
 #include <cstdint>
@@ -218,9 +218,12 @@ struct PsiFrag {
 };
 
 // C: tiles per block row, 1 or 2 with the pending sums of the backward sweep
-// in registers; 0: any c >= 3, pending sums in shared memory.
+// in registers; 0: any c >= 3, pending sums in shared memory.  Two column
+// fragments stay within 128 registers, two blocks of eight warps an SM (154
+// without the bound: 512^2 in 16^2 blocks x 32 97 us, with it 82); one (0: no bound) takes
+// what it needs, 80 to 118.
 template <typename TP, int NF, int MM, int C>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, NF == 2 ? 2 : 0)
 k_local_mma(const float* __restrict__ tiles_g, const SubInfo* __restrict__ subs,
             const int64_t* __restrict__ tile_off, const int64_t* __restrict__ brow0, const float* __restrict__ piv,
             const double* __restrict__ rin, const double* __restrict__ qin, const CgScalars* __restrict__ csc,
@@ -276,19 +279,16 @@ k_local_mma(const float* __restrict__ tiles_g, const SubInfo* __restrict__ subs,
         phase ^= 1u << slot;
         pend &= ~(1u << slot);
     };
-    const bool one = ld == 1;        // a single column: scalar accesses
-
     // r' = r - alpha q for this lane's columns of (system, rhs) pairs still iterating
     double al[NF][2];
-    bool up[NF][2], has[NF];
+    bool up[NF][2];
 #pragma unroll
     for (int nf = 0; nf < NF; ++nf) {
-        has[nf] = cb + 8 * nf + 2 * t < ld;      // below 8 right-hand sides the last columns are empty
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
             al[nf][j] = 0.0;
             up[nf][j] = false;
-            if (qin != nullptr && has[nf] && !(one && j == 1)) {
+            if (qin != nullptr) {
                 const CgScalars cs = csc[(int64_t)S.seg * ld + cb + 8 * nf + 2 * t + j];
                 up[nf][j] = cs.active != 0;
                 if (up[nf][j]) al[nf][j] = cs.alpha;
@@ -323,15 +323,10 @@ k_local_mma(const float* __restrict__ tiles_g, const SubInfo* __restrict__ subs,
             for (int nf = 0; nf < NF; ++nf) {
                 rraw[h][nf] = make_double2(0.0, 0.0);
                 qraw[h][nf] = make_double2(0.0, 0.0);
-                if (valid && has[nf]) {
+                if (valid) {
                     const int64_t e = e0 + (int64_t)row * ld + 8 * nf;
-                    if (one) {
-                        rraw[h][nf].x = rin[e];
-                        if (up[nf][0]) qraw[h][nf].x = qin[e];
-                    } else {
-                        rraw[h][nf] = *reinterpret_cast<const double2*>(rin + e);
-                        if (up[nf][0] || up[nf][1]) qraw[h][nf] = *reinterpret_cast<const double2*>(qin + e);
-                    }
+                    rraw[h][nf] = *reinterpret_cast<const double2*>(rin + e);
+                    if (up[nf][0] || up[nf][1]) qraw[h][nf] = *reinterpret_cast<const double2*>(qin + e);
                 }
             }
         }
@@ -343,11 +338,8 @@ k_local_mma(const float* __restrict__ tiles_g, const SubInfo* __restrict__ subs,
             if (row + row0 < n)
 #pragma unroll
                 for (int nf = 0; nf < NF; ++nf)
-                    if (has[nf]) {
-                        float* e = zf + e0 + (int64_t)row * ld + 8 * nf;
-                        if (one) *e = v[nf][2 * h];
-                        else *reinterpret_cast<float2*>(e) = make_float2(v[nf][2 * h], v[nf][2 * h + 1]);
-                    }
+                    *reinterpret_cast<float2*>(zf + e0 + (int64_t)row * ld + 8 * nf) =
+                        make_float2(v[nf][2 * h], v[nf][2 * h + 1]);
         }
     };
     // v = pivot * v + acc
@@ -462,7 +454,7 @@ k_local_mma(const float* __restrict__ tiles_g, const SubInfo* __restrict__ subs,
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const int mode = g + 8 * (i >> 1);
-                    if (mode < m && has[nf] && !(one && (i & 1)))
+                    if (mode < m)
                         rc[(S.coff + mode) * ld + cb + 8 * nf + 2 * t + (i & 1)] = racc[nf][i] + h1[(nf * 4 + i) * 32];
                 }
         pair_sync(group);
@@ -482,11 +474,8 @@ k_local_mma(const float* __restrict__ tiles_g, const SubInfo* __restrict__ subs,
             for (int nf = 0; nf < NF; ++nf) {
                 const int row = K * 32 + h;
                 yraw[h][nf] = make_float2(0.f, 0.f);
-                if (K >= 0 && row + row0 < n && has[nf]) {
-                    const float* e = zf + e0 + (int64_t)row * ld + 8 * nf;
-                    if (one) yraw[h][nf].x = *e;
-                    else yraw[h][nf] = *reinterpret_cast<const float2*>(e);
-                }
+                if (K >= 0 && row + row0 < n)
+                    yraw[h][nf] = *reinterpret_cast<const float2*>(zf + e0 + (int64_t)row * ld + 8 * nf);
             }
     };
     constexpr int NP = C > 0 ? C : 1;
@@ -619,12 +608,9 @@ void launch_pack_psi(cudaStream_t s, int nsub, const SubInfo* subs, const int64_
     }
 }
 
-// Columns a block computes: the right-hand sides, at least one MMA's eight.
-static int mma_cols(int ld) { return ld < 8 ? 8 : ld; }
-
 size_t local_mma_smem(int cmax, int ld, int depth) {
     const int nbuf = depth + 1;
-    return (size_t)nbuf * cmax * 4096 + (size_t)ring_bar_slots(nbuf) * 8 + (size_t)(cmax + 1) * mma_cols(ld) * 256;
+    return (size_t)nbuf * cmax * 4096 + (size_t)ring_bar_slots(nbuf) * 8 + (size_t)(cmax + 1) * ld * 256;
 }
 
 // Default ring depth: the deepest (at most 4) whose staging stays within
@@ -635,13 +621,10 @@ static int local_mma_depth(int cmax, int ld) {
     return d;
 }
 
-// One launch over all subdomains, or (a.nclass > 1) one per band-width
-// group with the ring sized for that width: narrow subdomains then take
-// less shared memory and more of their blocks share an SM.
 template <typename TP, int NF, int MM, int C>
 static cudaError_t mma_launch(const LocalTmaArgs& a, const void* psif, void* zf, void* rc, int nsub, int cmax,
                               int nbmax, const int32_t* order) {
-    const int warps = 2 * mma_cols(a.ld) / (8 * NF);
+    const int warps = 2 * a.ld / (8 * NF);
     auto kern = k_local_mma<TP, NF, MM, C>;
     static size_t smem_set = 0;
     // no deeper than the group's block rows: the rest of the ring would stay unused
@@ -659,21 +642,11 @@ static cudaError_t mma_launch(const LocalTmaArgs& a, const void* psif, void* zf,
 
 template <typename TP, int NF, int MM>
 static cudaError_t mma_nf(const LocalTmaArgs& a, const void* psif, void* zf, void* rc) {
-    auto launch = [&](int nsub, int cmax, int nbmax, const int32_t* order) -> cudaError_t {
-        // one band width per launch: nclass > 1 or all subdomains share cmax
+    return for_band_widths(a, [&](int nsub, int cmax, int nbmax, const int32_t* order) -> cudaError_t {
         if (cmax == 1) return mma_launch<TP, NF, MM, 1>(a, psif, zf, rc, nsub, cmax, nbmax, order);
         if (cmax == 2) return mma_launch<TP, NF, MM, 2>(a, psif, zf, rc, nsub, cmax, nbmax, order);
         return mma_launch<TP, NF, MM, 0>(a, psif, zf, rc, nsub, cmax, nbmax, order);
-    };
-    if (a.nclass <= 1 || a.order == nullptr) return launch(a.nsub, a.cmax, a.nbmax, nullptr);
-    const int32_t* ord = a.order;
-    for (int k = 0; k < a.nclass; ++k) {
-        if (a.class_n[k] == 0) continue;
-        const cudaError_t e = launch(a.class_n[k], a.class_c[k], a.class_nb[k], ord);
-        if (e != cudaSuccess) return e;
-        ord += a.class_n[k];
-    }
-    return cudaSuccess;
+    });
 }
 
 // Right-hand sides per column group: 8 (default), or 16 (a.nr).

@@ -17,7 +17,9 @@
 //   t = r_K - sum_d L_{K,K-c+d} y_{K-c+d} ;  y_K = L_KK^{-1} t
 // Backward sweep (lane = column l of block column K):
 //   w = y_K - sum_d L_{K+d,K}^T x_{K+d}   ;  x_K = L_KK^{-T} w
+#include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -424,6 +426,354 @@ k_local_tma1(const __grid_constant__ CUtensorMap tmF, const SubInfo* __restrict_
 }
 
 // ---------------------------------------------------------------------------
+// Two to four right-hand sides, and one on a subdomain too long for the kernel
+// above: W warps of NC columns each, lane = row (forward) or column (backward).
+//
+// All arithmetic is FP32 multiply-adds, each 32-term dot as four sums of packed
+// pairs.  Bound by the chain of dependent steps and the factor's bytes.  What was
+// there before: a lane per row with one sum a dot, forward and transposed tiles
+// and a ring of c + depth + 1 block rows (A); the MMA kernel with empty columns
+// (B), whose tensor cores truncate as they add up.  A / B / this, us a launch and
+// the FP32 apply's relative distance from the FP64 one on N(0, 1):
+//   1024^2 in 32^2 x 2  128 / 138 / 67    1.2e-7 / 2.7e-6 / 1.1e-7
+//   512^2 in 16^2 x 3    46 / 39 / 27     1.4e-7 / 5.8e-7 / 1.1e-7
+//   96x80x72 in 8^3 x 3 145 / 111 / 65    2.3e-7 / 6.8e-7 / 0.8e-7
+//   24^3 in 8^3 x 4      66 / 49 / 32     2.6e-7 / 5.8e-7 / 0.8e-7
+//   72^3 in 9^3 x 2     237 / 109 / 66    2.7e-7 / 1.1e-6 / 0.9e-7
+//   64,000 rows x 1    2281 / 2475 / 1337 1.9e-7 / 2.6e-6 / 0.8e-7
+// Four columns are one warp's or two warps' (a.nr): 65 / 67 us at 96x80x72, 41 / 33
+// at 24^3, 86 / 96 at 1024^2, 167 / 146 at 110^3; the tuner picks.
+//
+// The warps of a block share the ring of factor tiles only.  The backward sweep
+// is right-looking (see k_local_mma.cu): step K adds the transposes of its own
+// block row's tiles times x_K to the pending sums of block rows K-1..K-c, so the
+// ring is depth + 1 block rows and a subdomain's y may have any length (it waits
+// in z_f).  C: tiles per block row, 1 or 2 with the pending sums in registers;
+// 0: any c >= 3, pending sums in shared memory.
+// ---------------------------------------------------------------------------
+// NC consecutive values of a row (8-byte aligned for NC = 1, 16 for more).
+template <int NC>
+__device__ __forceinline__ void load_cols(const double* p, double (&v)[NC]) {
+    if constexpr (NC == 1) {
+        v[0] = *p;
+    } else {
+#pragma unroll
+        for (int j = 0; j < NC; j += 2) {
+            const double2 d = *reinterpret_cast<const double2*>(p + j);
+            v[j] = d.x;
+            v[j + 1] = d.y;
+        }
+    }
+}
+template <int NC>
+__device__ __forceinline__ void load_cols(const float* p, float (&v)[NC]) {
+    if constexpr (NC == 4) {
+        const float4 d = *reinterpret_cast<const float4*>(p);
+        v[0] = d.x, v[1] = d.y, v[2] = d.z, v[3] = d.w;
+    } else if constexpr (NC == 2) {
+        const float2 d = *reinterpret_cast<const float2*>(p);
+        v[0] = d.x, v[1] = d.y;
+    } else {
+        v[0] = *p;
+    }
+}
+template <int NC>
+__device__ __forceinline__ void store_cols(float* p, const float (&v)[NC]) {
+    if constexpr (NC == 4) *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    else if constexpr (NC == 2) *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
+    else *p = v[0];
+}
+// Row `lane` of a swizzled tile as 16 column pairs.
+__device__ __forceinline__ void row_pairs(const float* T, const int (&rsw)[8], float2 (&a)[16]) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const float4 m4 = *reinterpret_cast<const float4*>(T + rsw[j]);
+        a[2 * j] = lo2(m4);
+        a[2 * j + 1] = hi2(m4);
+    }
+}
+
+template <typename TP, int NC, int W, int MM, int C>
+__global__ void __launch_bounds__(32 * W, 8)
+k_local_few(const __grid_constant__ CUtensorMap tmF, const SubInfo* __restrict__ subs,
+            const int64_t* __restrict__ tile_row0, const float* __restrict__ piv, const double* __restrict__ rin,
+            const double* __restrict__ qin, const CgScalars* __restrict__ csc, float* __restrict__ zf,
+            const TP* __restrict__ psi, float* __restrict__ rc, int ld, int cmax, int depth, int64_t budget,
+            SolveState* st, int32_t* err, int probe, const int32_t* __restrict__ order) {
+    pdl_wait();
+    if (st != nullptr && st->done) return;
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char* base = smem_align1024(smem_raw);
+    const int sid = order != nullptr ? order[blockIdx.x] : (int)blockIdx.x;
+    const SubInfo S = subs[sid];
+    if (!AMS_ROW_OK(S.row0, 5) || !AMS_ROW_OK(S.row0 + S.n - 1, 5)) return;
+    const int c = C > 0 ? C : S.c, cs = C > 0 ? C : cmax;
+    const int nb = S.nb, n = S.n, m = S.m;
+    const int D = depth, nbuf = D + 1;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, cb = warp * NC;
+    constexpr int BF = 32 * NC;                                // floats of a block [column][row]
+    float* tiles = (float*)base;                               // nbuf * cs * 1024
+    uint64_t* bars = (uint64_t*)(tiles + (size_t)nbuf * cs * 1024);
+    // per warp: a block for t and w, a ring of cs blocks for y (block 0 then holds x), and pending blocks when C = 0
+    float* tmp = (float*)(bars + ring_bar_slots(nbuf)) + (size_t)warp * BF * (1 + cs + (C > 0 ? 0 : cs));
+    float* yr = tmp + BF;
+    float* pw = yr + (size_t)cs * BF + lane;
+    const int64_t trow = tile_row0[sid];
+    const uint32_t row_bytes = 4096u * (uint32_t)c;
+    uint32_t phase = 0, pend = 0;    // change only when a wait succeeds: the exit drain finds every copy in flight
+    bool ok = true;
+
+    int rsw[8], csw[8];
+    float2 mk[16];                   // forward: 1 where column >= lane; backward: 1 where row > lane
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        rsw[j] = lane * 32 + ((j ^ (lane & 7)) << 2);               // chunk j of tile row `lane`
+        csw[j] = (((lane >> 2) ^ j) << 2) + (lane & 3);             // element (r, lane) sits at r * 32 + csw[r & 7]
+    }
+#pragma unroll
+    for (int i = 0; i < 16; ++i) mk[i] = make_float2(2 * i >= lane ? 1.f : 0.f, 2 * i + 1 >= lane ? 1.f : 0.f);
+    const float2 neg1 = make_float2(-1.f, -1.f);
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i <= nbuf; ++i) mbar_init(smem_u32(bars + i), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    __syncthreads();
+    auto issue = [&](int K, int slot) {
+        if (threadIdx.x == 0) {
+            const uint32_t bar = smem_u32(bars + slot);
+            mbar_expect_tx(bar, row_bytes);
+            for (int d = 0; d < c; ++d)
+                tma_load_2d(smem_u32(tiles + ((size_t)slot * cs + d) * 1024), &tmF, 0,
+                            (int32_t)(trow + ((int64_t)K * c + d) * 32), bar);
+        }
+        pend |= 1u << slot;
+    };
+    auto wait_slot = [&](int slot) {
+        if (!mbar_wait(smem_u32(bars + slot), (phase >> slot) & 1u, budget)) {
+            ok = false;
+            return;
+        }
+        phase ^= 1u << slot;
+        pend &= ~(1u << slot);
+    };
+
+    // r' = r - alpha q for this warp's columns of (system, rhs) pairs still iterating
+    double al[NC];
+    bool up[NC], any = false;
+#pragma unroll
+    for (int j = 0; j < NC; ++j) {
+        al[j] = 0.0;
+        up[j] = false;
+        if (qin != nullptr) {
+            const CgScalars cj = csc[(int64_t)S.seg * ld + cb + j];
+            up[j] = cj.active != 0;
+            if (up[j]) al[j] = cj.alpha;
+        }
+        any = any || up[j];
+    }
+    float2 racc[NC][MM / 2];
+#pragma unroll
+    for (int j = 0; j < NC; ++j)
+#pragma unroll
+        for (int k = 0; k < MM / 2; ++k) racc[j][k] = make_float2(0.f, 0.f);
+
+    // Inputs of a block row are loaded PF steps ahead, alternating registers (one where two warps take 128 registers).
+    constexpr int PF = W == 1 ? 2 : 1;
+    const int64_t e0 = (S.row0 + lane) * ld + cb;
+    const bool vec = m == MM && (reinterpret_cast<uintptr_t>(psi + S.psi_off) & 15) == 0;
+    double rn[PF][NC], qn[PF][NC];
+    BasisRow<TP, MM> bn[PF];
+    float pv[PF], yn[PF][NC];
+    auto load_piv = [&](int K, float& p) {
+        const int row = K * 32 + lane;
+        p = 1.f;
+        if (K >= 0 && row < n) p = __ldg(piv + S.row0 + row);
+    };
+    auto load_in = [&](int K, int u) {
+        const int row = K * 32 + lane;
+#pragma unroll
+        for (int j = 0; j < NC; ++j) rn[u][j] = qn[u][j] = 0.0;
+        bn[u].clear();
+        load_piv(K < nb ? K : nb - 1, pv[u]);
+        if (K < nb && row < n) {
+            load_cols<NC>(rin + e0 + (int64_t)K * 32 * ld, rn[u]);
+            if (any) load_cols<NC>(qin + e0 + (int64_t)K * 32 * ld, qn[u]);
+            if (rc != nullptr) bn[u].load(psi + S.psi_off + (int64_t)row * m, m, vec);
+        }
+    };
+    auto store_z = [&](int K, const float (&v)[NC]) {
+        if (K * 32 + lane < n) store_cols<NC>(zf + e0 + (int64_t)K * 32 * ld, v);
+    };
+
+    for (int j = 0; j < D && j < nb; ++j) issue(j, j);
+    if (probe) {   // timeout test hook: a bounded wait on a barrier nothing completes
+        if (!mbar_wait(smem_u32(bars + nbuf), 0u, budget)) ok = false;
+        ok = __syncthreads_and(ok);
+    }
+#pragma unroll
+    for (int u = 0; u < PF; ++u) load_in(u, u);
+    int sK = 0, sI = D;              // slots of block rows K and K + D
+    int yK = 0;                      // K mod c
+
+    // ---------------- forward ----------------
+    // t = r'_K - sum_d L_{K,K-c+d} y_{K-c+d}, y_K = L_KK^{-1} t; y_K takes the ring block of y_{K-c}
+    auto fwd_step = [&](int K, int u) {
+        float t[NC];
+#pragma unroll
+        for (int j = 0; j < NC; ++j) {
+            t[j] = __double2float_rn(up[j] ? fma(-al[j], qn[u][j], rn[u][j]) : rn[u][j]);
+            if (rc != nullptr) {
+                const float2 t2 = make_float2(t[j], t[j]);
+#pragma unroll
+                for (int k = 0; k < MM / 2; ++k) racc[j][k] = __ffma2_rn(bn[u].get2(k), t2, racc[j][k]);
+            }
+        }
+        const float p = pv[u];
+        load_in(K + PF, u);
+        wait_slot(sK);
+        const float* T = tiles + (size_t)sK * cs * 1024;
+        if (C != 1)
+#pragma unroll 1
+            for (int d = 1; d < c; ++d) {
+                const int src = K - c + d;
+                if (src < 0) continue;
+                float2 a[16];
+                row_pairs(T + d * 1024, rsw, a);
+                const float* v = yr + (C == 2 ? yK ^ 1 : src % c) * BF;
+#pragma unroll
+                for (int j = 0; j < NC; ++j) t[j] -= pdot16(a, v + 32 * j);
+            }
+        float2 a[16];                // row `lane` of M_K: columns >= lane (L_{K,K-c}), then columns < lane (L_KK^{-1})
+        if (K >= c) {
+            row_pairs(T, rsw, a);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) a[i] = __fmul2_rn(a[i], mk[i]);
+#pragma unroll
+            for (int j = 0; j < NC; ++j) t[j] -= pdot16(a, yr + yK * BF + 32 * j);
+        }
+#pragma unroll
+        for (int j = 0; j < NC; ++j) tmp[32 * j + lane] = t[j];
+        ok = __syncthreads_and(ok);  // t is there; every warp is past block row K - 1
+        if (!ok) return;
+        if (K + D < nb) issue(K + D, sI);
+        row_pairs(T, rsw, a);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) a[i] = __ffma2_rn(__fmul2_rn(a[i], mk[i]), neg1, a[i]);
+#pragma unroll
+        for (int j = 0; j < NC; ++j) {
+            t[j] = fmaf(p, t[j], pdot16(a, tmp + 32 * j));
+            yr[yK * BF + 32 * j + lane] = t[j];
+        }
+        store_z(K, t);
+        sK = sK + 1 == nbuf ? 0 : sK + 1;
+        sI = sI + 1 == nbuf ? 0 : sI + 1;
+        yK = yK + 1 == c ? 0 : yK + 1;
+        __syncwarp();                // y_K is there; t is no longer read
+    };
+#pragma unroll 1
+    for (int K = 0; K < nb && ok; K += PF) {
+        fwd_step(K, 0);
+        if (PF == 2 && K + 1 < nb && ok) fwd_step(K + 1, PF - 1);
+    }
+    if (rc != nullptr && ok) {
+#pragma unroll
+        for (int j = 0; j < NC; ++j)
+#pragma unroll
+            for (int k = 0; k < MM; ++k) {
+                float v = (k & 1) ? racc[j][k / 2].y : racc[j][k / 2].x;
+                for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+                if (lane == 0 && k < m) rc[(S.coff + k) * ld + cb + j] = v;
+            }
+    }
+    pdl_trigger();
+
+    // ---------------- backward ----------------
+    // w = y_K - pending_K, x_K = L_KK^{-T} w, pending_{K-c+d} += L_{K,K-c+d}^T x_K; block rows nb - nbuf .. nb - 1 are
+    // still in the ring, y of a step (written by this lane) is loaded PF steps ahead
+    const int Rres = nb > nbuf ? nb - nbuf : 0;
+    auto load_back = [&](int K, int u) {
+#pragma unroll
+        for (int j = 0; j < NC; ++j) yn[u][j] = 0.f;
+        load_piv(K, pv[u]);
+        if (K >= 0 && K * 32 + lane < n) load_cols<NC>(zf + e0 + (int64_t)K * 32 * ld, yn[u]);
+    };
+#pragma unroll
+    for (int i = 0; i < 16; ++i) mk[i] = make_float2(2 * i > lane ? 1.f : 0.f, 2 * i + 1 > lane ? 1.f : 0.f);
+    constexpr int NP = C > 0 ? C : 1;
+    float pnd[NP][NC];               // C > 0: pending sums of block rows K, K - 1
+#pragma unroll
+    for (int j = 0; j < NC; ++j) pnd[0][j] = pnd[NP - 1][j] = 0.f;
+    if (C == 0)
+        for (int i = 0; i < c * NC; ++i) pw[32 * i] = 0.f;
+    if (ok) {
+#pragma unroll
+        for (int u = 0; u < PF; ++u) load_back(nb - 1 - u, u);
+    }
+    sK = (nb - 1) % nbuf;
+    auto bwd_step = [&](int K, int u) {
+        float w[NC];
+#pragma unroll
+        for (int j = 0; j < NC; ++j) {
+            float* e = pw + ((size_t)(K % c) * NC + j) * 32;
+            w[j] = yn[u][j] - (C > 0 ? pnd[0][j] : *e);
+            if (C == 0) *e = 0.f;
+            tmp[32 * j + lane] = w[j];
+        }
+        const float p = pv[u];
+        load_back(K - PF, u);
+        if (K < Rres) wait_slot(sK);
+        ok = __syncthreads_and(ok);  // w is there; every warp is past block row K + 1
+        if (!ok) return;
+        if (K - D >= 0 && K - D < Rres) issue(K - D, sK + 1 == nbuf ? 0 : sK + 1);   // into its slot
+        const float* T = tiles + (size_t)sK * cs * 1024;
+        float2 a[16];                // column `lane` of M_K: rows > lane (L_KK^{-1}), then rows <= lane (L_{K,K-c})
+        col_pairs(T, csw, a);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) a[i] = __fmul2_rn(a[i], mk[i]);
+#pragma unroll
+        for (int j = 0; j < NC; ++j) {
+            w[j] = fmaf(p, w[j], pdot16(a, tmp + 32 * j));
+            yr[32 * j + lane] = w[j];
+        }
+        store_z(K, w);
+        __syncwarp();                // x_K is there; w is no longer read
+        col_pairs(T, csw, a);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) a[i] = __ffma2_rn(__fmul2_rn(a[i], mk[i]), neg1, a[i]);
+        if constexpr (C > 0) {
+#pragma unroll
+            for (int j = 0; j < NC; ++j) {
+                pnd[0][j] = pnd[C - 1][j];
+                pnd[C - 1][j] = pdot16(a, yr + 32 * j);
+            }
+            if (C == 2) {
+                col_pairs(T + 1024, csw, a);
+#pragma unroll
+                for (int j = 0; j < NC; ++j) pnd[0][j] += pdot16(a, yr + 32 * j);
+            }
+        } else {
+#pragma unroll 1
+            for (int d = 0; d < c; ++d) {
+                const int dst = K - c + d;
+                if (d > 0) col_pairs(T + d * 1024, csw, a);
+                if (dst < 0) continue;
+                float* e = pw + (size_t)(dst % c) * BF;
+#pragma unroll
+                for (int j = 0; j < NC; ++j) e[32 * j] += pdot16(a, yr + 32 * j);
+            }
+        }
+        sK = sK == 0 ? nbuf - 1 : sK - 1;
+    };
+#pragma unroll 1
+    for (int K = nb - 1; K >= 0 && ok; K -= PF) {
+        bwd_step(K, 0);
+        if (PF == 2 && K >= 1 && ok) bwd_step(K - 1, PF - 1);
+    }
+    if (!ok) timeout_drain(bars, nbuf, pend, phase, err, st, threadIdx.x == 0);
+}
+
+// ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
 size_t local_tma1_smem(int cmax, int nbmax, int depth) {
@@ -457,21 +807,67 @@ static cudaError_t tma1(const LocalTmaArgs& a, const void* psi, void* zf, void* 
                          a.l2mode, a.l2keep, a.budget, a.st, a.err, a.probe);
 }
 
+// Staging of the few-column kernel: ring, barriers, and per column the blocks of t, y and (from three tiles) pending sums.
+static size_t local_few_smem(int cmax, int ld, int depth) {
+    const int nbuf = depth + 1;
+    return 1024 /* alignment slack */ + (size_t)nbuf * cmax * 4096 + (size_t)ring_bar_slots(nbuf) * 8 +
+           (size_t)ld * 128 * (1 + cmax + (cmax > 2 ? cmax : 0));
+}
+
+template <typename TP, int NC, int W, int MM, int C>
+static cudaError_t few_launch(const LocalTmaArgs& a, const void* psi, void* zf, void* rc, int nsub, int cmax, int nbmax,
+                              const int32_t* order) {
+    auto kern = k_local_few<TP, NC, W, MM, C>;
+    int depth = a.depth > 0 ? a.depth : 4;
+    if (a.depth == 0)
+        while (depth > 2 && local_few_smem(cmax, a.ld, depth) > 28 * 1024) --depth;
+    depth = std::max(1, std::min(depth, nbmax));   // the rest of the ring would stay unused
+    const size_t smem = local_few_smem(cmax, a.ld, depth);
+    static size_t smem_set = 0;
+    if (smem > smem_set) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        smem_set = smem;
+    }
+    return launch_kernel(a.pdl, kern, dim3(nsub), dim3(32 * W), smem, a.stream, *a.tmF, a.subs, a.tile_row0, a.piv,
+                         a.in.r, a.in.q, a.in.sc, (float*)zf, (const TP*)psi, (float*)rc, a.ld, cmax, depth, a.budget, a.st, a.err, a.probe, order);
+}
+template <typename TP, int NC, int W>
+static cudaError_t few_nc(const LocalTmaArgs& a, const void* psi, void* zf, void* rc) {
+    return for_band_widths(a, [&](int nsub, int cmax, int nbmax, const int32_t* order) -> cudaError_t {
+        auto mm = [&](auto M) -> cudaError_t {
+            constexpr int MM = decltype(M)::value;
+            if (cmax == 1) return few_launch<TP, NC, W, MM, 1>(a, psi, zf, rc, nsub, cmax, nbmax, order);
+            if (cmax == 2) return few_launch<TP, NC, W, MM, 2>(a, psi, zf, rc, nsub, cmax, nbmax, order);
+            return few_launch<TP, NC, W, MM, 0>(a, psi, zf, rc, nsub, cmax, nbmax, order);
+        };
+        return a.mmax > 8 ? mm(std::integral_constant<int, 16>{}) : mm(std::integral_constant<int, 8>{});
+    });
+}
+// Columns a warp: all of them (a.nr = 4, or two columns), or two of four.
+template <typename TP>
+static cudaError_t few_tp(const LocalTmaArgs& a, const void* psi, void* zf, void* rc) {
+    if (a.ld == 1) return few_nc<TP, 1, 1>(a, psi, zf, rc);
+    if (a.ld == 2) return few_nc<TP, 2, 1>(a, psi, zf, rc);
+    return a.nr == 4 ? few_nc<TP, 4, 1>(a, psi, zf, rc) : few_nc<TP, 2, 2>(a, psi, zf, rc);
+}
+
 // The one-right-hand-side kernel keeps y for a whole subdomain in shared
-// memory; larger subdomains and more right-hand sides use the MMA kernel.
-// (At 3 right-hand sides, 96x80x72 cells in 8^3 blocks, a row-per-lane FP32
-// kernel took 152 us a launch, the MMA kernel with five of its eight
-// columns empty 117 us.)
-static bool use_tma1(const LocalTmaArgs& a) {
+// memory; longer subdomains and two to four right-hand sides use the few-column
+// kernel (both sides of that line are measured there), more the MMA kernel.
+bool local_one_vector(const LocalTmaArgs& a) {
     return a.ld == 1 && local_tma1_smem(a.cmax, a.nbmax, 2) <= 200 * 1024;
 }
 
 size_t local_tma_launch_smem(const LocalTmaArgs& a, int depth) {
-    return use_tma1(a) ? local_tma1_smem(a.cmax, a.nbmax, depth) : local_mma_smem(a.cmax, a.ld, depth);
+    if (local_one_vector(a)) return local_tma1_smem(a.cmax, a.nbmax, depth);
+    return a.ld <= 4 ? local_few_smem(a.cmax, a.ld, depth) : local_mma_smem(a.cmax, a.ld, depth);
 }
 
 cudaError_t launch_local_tma(const LocalTmaArgs& a, int prec, const void* psi, const void* psif, void* zf, void* rc) {
-    if (!use_tma1(a)) return launch_local_mma(a, prec, psif, zf, rc);
+    if (a.ld > 4) return launch_local_mma(a, prec, psif, zf, rc);
+    if (!local_one_vector(a))
+        return prec == AMS_PREC_FP32 ? few_tp<float>(a, psi, zf, rc) : few_tp<__nv_bfloat16>(a, psi, zf, rc);
     const bool big = a.mmax > 8, c1 = a.cmax == 1;
     if (prec == AMS_PREC_FP32) {
         if (big) return c1 ? tma1<float, 16, true>(a, psi, zf, rc) : tma1<float, 16, false>(a, psi, zf, rc);

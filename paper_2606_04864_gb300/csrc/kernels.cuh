@@ -66,7 +66,7 @@ template <> __device__ __forceinline__ double from_d<double>(double v) { return 
 // time in the checking build.  In the release build the checks compile to
 // `true` and the hooks do nothing.
 // Sites: 1 SpMV column, 2 prolongation gather of y, 3 coarse-product
-// gather, 4 several-RHS local solve rows, 5 one-RHS local solve rows,
+// gather, 4 local solve rows from five right-hand sides on, 5 up to four,
 // 6 caller-order permutation, 99 the self-test.
 // ---------------------------------------------------------------------------
 struct DebugBounds {

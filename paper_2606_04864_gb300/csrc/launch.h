@@ -94,21 +94,37 @@ struct LocalTmaArgs {
     SolveState* st;
     bool pdl;
     int depth;               // ring depth (block rows in flight); 0: chosen from the band width
-    int nr;                  // several-RHS kernel: right-hand sides per warp (8, or 16 from 16 on); else default
+    int nr;                  // right-hand sides per warp (2 to 4: 2 or 4) or per two warps (from 5: 8 or 16); 0: default
     int l2mode;              // one-RHS kernel, L2 priority of factor tiles: 0 none, 1 evict-first on
                              // tiles read for the last time, 2 as 1 plus evict-last on kept tiles
     int l2keep;              // block rows below the ring's resident ones whose forward load is
                              // kept (not marked evict-first): the backward sweep reloads them soonest
     int32_t* err;            // status word set to AMS_ERR_DEVICE_TIMEOUT when a wait runs out (or NULL)
     int probe;               // 1: every block first waits on a barrier nothing completes (timeout test)
-    // several-RHS kernel: subdomains grouped by band width, one launch per
-    // group sized for its own width (nclass <= 1: one launch over all)
+    // all but the one-vector kernel: subdomains grouped by band width (see
+    // for_band_widths; nclass <= 1: one launch over all)
     int nclass = 0;
     const int* class_c = nullptr;        // host: band tiles of each group
     const int* class_n = nullptr;        // host: subdomains of each group
     const int* class_nb = nullptr;       // host: most block rows of a subdomain in each group
     const int32_t* order = nullptr;      // device: subdomain ids, group after group
 };
+// launch(subdomains, band tiles, most block rows, order) over all subdomains, or
+// (a.nclass > 1) once per band-width group with the staging sized for that
+// width: narrow subdomains then take less shared memory and more of their
+// blocks share an SM.  Every launch has one band width.
+template <typename F>
+inline cudaError_t for_band_widths(const LocalTmaArgs& a, const F& launch) {
+    if (a.nclass <= 1 || a.order == nullptr) return launch(a.nsub, a.cmax, a.nbmax, (const int32_t*)nullptr);
+    const int32_t* ord = a.order;
+    for (int k = 0; k < a.nclass; ++k) {
+        if (a.class_n[k] == 0) continue;
+        const cudaError_t e = launch(a.class_n[k], a.class_c[k], a.class_nb[k], ord);
+        if (e != cudaSuccess) return e;
+        ord += a.class_n[k];
+    }
+    return cudaSuccess;
+}
 
 struct CoarseLaunch {
     cudaStream_t stream;
@@ -136,9 +152,11 @@ size_t local_solve_smem(int cmax, int ld, size_t tf_bytes, int depth);
 // FP64 local solves (k_local_f64.cu)
 cudaError_t launch_local_solve(const LocalSolveArgs& a, const double* fac, const double* psi, double* zf, double* rc);
 void launch_coarse_gemm(const CoarseLaunch& c, int prec, int ld, const void* in, void* out);
+// The launch uses the one-vector kernel (one launch whatever the band widths).
+bool local_one_vector(const LocalTmaArgs& a);
 // psif: the basis in fragment order (launch_pack_psi), read by the MMA kernel
 cudaError_t launch_local_tma(const LocalTmaArgs& a, int prec, const void* psi, const void* psif, void* zf, void* rc);
-// several right-hand sides: tile products as tensor-core MMAs (k_local_mma.cu)
+// from five right-hand sides on: tile products as tensor-core MMAs (k_local_mma.cu)
 cudaError_t launch_local_mma(const LocalTmaArgs& a, int prec, const void* psif, void* zf, void* rc);
 size_t local_mma_smem(int cmax, int ld, int depth);
 // Basis in MMA fragment order: 16-byte words per block row, and the packing

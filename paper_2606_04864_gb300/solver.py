@@ -108,10 +108,10 @@ class _Base:
     def launch_shape(self, nrhs: int = 1) -> dict:
         """Launch shapes used for solves with `nrhs` right-hand sides: blocks
         per SM of the element and subdomain grids, local-solve ring depth
-        (0 = derived from the band width), right-hand sides per warp of the
-        several-RHS local solve (0 = default), L2 priorities of the one-RHS
-        local solve's tile copies (mode 0/1/2 and kept block rows), and
-        whether they are fixed."""
+        (0 = derived from the band width), right-hand sides per warp (up to
+        four) or per two warps (more) of the local solve (0 = default), L2
+        priorities of the one-RHS local solve's tile copies (mode 0/1/2 and
+        kept block rows), and whether they are fixed."""
         a = np.zeros(7, dtype=np.int32)
         check(lib().ams_get_launch_shape(self._h, int(nrhs), _ptr(a)), "ams_get_launch_shape")
         d = dict(zip(self._SHAPE_KEYS, (int(v) for v in a[:6])))
