@@ -148,7 +148,7 @@ k_coarse_gemm(const CoarseItem* __restrict__ items, const TF* __restrict__ mat,
 // Many right-hand sides (LD >= 8) in the reduced-precision apply: the same
 // items as k_coarse_gemm, with the 32-row tile times the gathered input
 // computed by warp-level tensor-core MMAs (m16n8k8, TF32 head/tail split
-// of both operands, FP32 accumulation: FP32 accuracy).  Every warp computes
+// of both operands, FP32 accumulation, mma_tf32.cuh).  Every warp computes
 // the whole 32 x LD output tile over its own k-steps of each stage (warp w
 // takes k-steps w, w + NW, ..; NW = LD/4 warps), so each staged element is
 // split into its TF32 head and tail exactly once; the warps' partial tiles
