@@ -535,8 +535,10 @@ static ams_status setup_eigen(ams_handle h, const int64_t* d_rowptr, const int32
     // factor offsets are reused because the band structure is identical
     AMS_TRY(build_local_factors(h, d_rowptr, d_colind, d_vals, d_S, d_ahat, sigma, 1, &d_efac, &efac_elems, 1));
     double *d_X = nullptr, *d_Y = nullptr, *d_AY = nullptr, *d_T = nullptr, *d_theta = nullptr,
-           *d_res = nullptr;
+           *d_res = nullptr, *d_gap = nullptr;
     int32_t* d_status = nullptr;
+    const std::vector<double> no_gap(2 * (size_t)h->N, 1.0);   // see k_eig_resid
+    AMS_TRY(upload(h, &d_gap, no_gap));
     AMS_TRY(h->alloc_t(&d_X, (size_t)h->n_pad * P));
     AMS_TRY(h->alloc_t(&d_Y, (size_t)h->n_pad * P));
     AMS_TRY(h->alloc_t(&d_AY, (size_t)h->n_pad * P));
@@ -575,9 +577,10 @@ static ams_status setup_eigen(ams_handle h, const int64_t* d_rowptr, const int32
         return AMS_OK;
     };
     // Degree of the next filter: with T = (Ahat + sigma S)^{-1} S and per
-    // subdomain mu = 1 / (theta_p + sigma), the smallest Ritz value of T in
-    // the block, T_d(2 T / mu - 1) keeps the components below mu (the ones to
-    // be damped) within 1 and grows those above it like cosh(d acosh(.)):
+    // subdomain mu = 1 / (g (theta_p + sigma)), the smallest Ritz value of T in
+    // the block by the gap g (k_eig_resid; 1 at first), T_d(2 T / mu - 1) keeps the
+    // components below mu (the ones to be damped) within 1 and grows those above it
+    // like cosh(d acosh(.)); with a large g it is a plain power.  With g = 1
     // a plain step multiplies an eigenvector by its ratio to mu, the filter by
     // about the square of twice that ratio per two steps.  The number of
     // solves to 1e-13 falls from 48-68 to 25-34 (8^3 blocks, m = 6).  The
@@ -598,15 +601,15 @@ static ams_status setup_eigen(ams_handle h, const int64_t* d_rowptr, const int32
         d = std::min(d, maxit - it + 1);
         AMS_TRY(solve(d_X, d_Y));
         if (d > 1) {
-            launch_eig_cheb(h->stream, h->n_pad, P, h->d_sub_of_row, d_esubs, d_theta, sigma, 2.0, d_Y, 0.0, nullptr, 1.0,
-                            d_X, d_Y);                                      // T_1
+            launch_eig_cheb(h->stream, h->n_pad, P, h->d_sub_of_row, d_esubs, d_theta, d_gap, sigma, 2.0, d_Y, 0.0, nullptr,
+                            1.0, d_X, d_Y);                                      // T_1
             AMS_TRY(solve(d_Y, d_AY));
             double *t2 = d == 2 ? d_Y : d_AY, *t3 = d_Y;
-            launch_eig_cheb(h->stream, h->n_pad, P, h->d_sub_of_row, d_esubs, d_theta, sigma, 4.0, d_AY, 2.0, d_Y, 1.0,
+            launch_eig_cheb(h->stream, h->n_pad, P, h->d_sub_of_row, d_esubs, d_theta, d_gap, sigma, 4.0, d_AY, 2.0, d_Y, 1.0,
                             d_X, t2);                                       // T_2
             if (d == 3) {
                 AMS_TRY(solve(d_AY, d_X));
-                launch_eig_cheb(h->stream, h->n_pad, P, h->d_sub_of_row, d_esubs, d_theta, sigma, 4.0, d_X, 2.0, d_AY,
+                launch_eig_cheb(h->stream, h->n_pad, P, h->d_sub_of_row, d_esubs, d_theta, d_gap, sigma, 4.0, d_X, 2.0, d_AY,
                                 1.0, d_Y, t3);                              // T_3
             }
             it += d - 1;
@@ -620,7 +623,7 @@ static ams_status setup_eigen(ams_handle h, const int64_t* d_rowptr, const int32
         AMS_CUDA_TRY(cudaGetLastError());
         if (check) {
             launch_eig_resid(h->stream, h->N, d_esubs, P, d_rowptr, d_colind, d_vals, d_S, d_ahat, d_X, d_theta,
-                             ncheck, sigma, d_res);
+                             ncheck, sigma, d > 1 ? d : 0, d_gap, d_res);
             AMS_CUDA_TRY(cudaMemcpyAsync(res.data(), d_res, sizeof(double) * res.size(), cudaMemcpyDeviceToHost,
                                          h->stream));
             AMS_CUDA_TRY(cudaStreamSynchronize(h->stream));
@@ -635,7 +638,7 @@ static ams_status setup_eigen(ams_handle h, const int64_t* d_rowptr, const int32
     launch_eig_update(h->stream, h->n_pad, P, h->d_sub_of_row, d_esubs, d_X, d_T, d_Y);
     std::swap(d_X, d_Y);
     launch_eig_resid(h->stream, h->N, d_esubs, P, d_rowptr, d_colind, d_vals, d_S, d_ahat, d_X, d_theta,
-                     ncheck, sigma, d_res);
+                     ncheck, sigma, 0, d_gap, d_res);
     std::vector<double> theta((size_t)h->N * P);
     int32_t status = 0;
     AMS_CUDA_TRY(cudaMemcpyAsync(theta.data(), d_theta, sizeof(double) * theta.size(), cudaMemcpyDeviceToHost,
@@ -682,7 +685,7 @@ static ams_status setup_eigen(ams_handle h, const int64_t* d_rowptr, const int32
     AMS_CUDA_TRY(cudaGetLastError());
     AMS_CUDA_TRY(cudaStreamSynchronize(h->stream));
     for (void* p : {(void*)d_S, (void*)d_ahat, d_efac, (void*)d_X, (void*)d_Y, (void*)d_AY, (void*)d_T,
-                    (void*)d_theta, (void*)d_res})
+                    (void*)d_theta, (void*)d_res, (void*)d_gap})
         h->release(p);
     h->info.eig_seconds = now_s() - t0;
     return AMS_OK;

@@ -561,30 +561,46 @@ __global__ void k_eig_update(int64_t nrows_pad, int P, const int32_t* __restrict
 }
 
 // One step of the Chebyshev recurrence of the filtered subspace iteration, per
-// row of a subdomain with largest Ritz value theta_p:
-//   out = k (theta_p + sigma) w - a u - b v   (u may be NULL; out may be w, u or v)
+// row of a subdomain with largest Ritz value theta_p and gap g (k_eig_resid):
+//   out = k g (theta_p + sigma) w - a u - b v   (u may be NULL; out may be w, u or v)
 __global__ void k_eig_cheb(int64_t nrows_pad, int P, const int32_t* __restrict__ sub_of_row,
-                           const SubInfo* __restrict__ subs, const double* __restrict__ theta, double sigma, double k,
-                           const double* w, double a, const double* u, double b, const double* v, double* out) {
+                           const SubInfo* __restrict__ subs, const double* __restrict__ theta,
+                           const double* __restrict__ gap, double sigma, double k, const double* w, double a,
+                           const double* u, double b, const double* v, double* out) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= nrows_pad * P) return;
     const int s = sub_of_row[t / P];
     if (s < 0) return;
-    const double f = k * (theta[(int64_t)s * P + subs[s].p - 1] + sigma);
+    const double f = k * gap[s] * (theta[(int64_t)s * P + subs[s].p - 1] + sigma);
     double x = fma(f, w[t], -b * v[t]);
     if (u != nullptr) x = fma(-a, u[t], x);
     out[t] = x;
 }
 
 // residual norms ||\hat A x_k - theta_k S x_k||_{S^{-1}} for k < ncheck into
-// resid[0 .. nsub), and the spread (theta_p + sigma) / (theta_1 + sigma) of
+// resid[0 .. nsub), and the spread g (theta_p + sigma) / (theta_1 + sigma) of
 // the shifted Ritz values into resid[nsub .. 2 nsub) (infinite where the
-// lowest is not positive: the shift does not make the pencil definite there)
+// lowest is not positive: the shift does not make the pencil definite there).
+//
+// gap[0 .. nsub): by how much the eigenvalues outside the block are taken to lie
+// above theta_p: the filter damps mu / g and below; [nsub .. 2 nsub): may it rise.  With the block's edge
+// inside a cluster (as many high-contrast islands as columns) the interval below
+// mu itself holds nothing but a distant rest, which the polynomial then keeps as
+// it is where plain steps would damp it: 16 islands of 1e6 in a 32^2 block, 6
+// modes, did not converge in 300 solves where plain steps take 40.  So, after a
+// filter step of degree d (0: none since the last call), whose guaranteed
+// reduction is gr = T_d(2 g (theta_p + sigma) / (theta_k + sigma) - 1): a residual
+// that fell by less than gr was held up from above mu / g, which tells g; one
+// that fell by gr or more, with gr below 2 a solve, doubles it, until it once
+// came back below 1.5 (the cluster goes on past the block: 25 islands, 9 modes,
+// 32 columns 85 solves at g = 1, 100 with a g that keeps rising, 88 so).  The 16
+// islands above: 28 solves.
+constexpr double kMaxGap = 64.0;
 __global__ void k_eig_resid(const SubInfo* __restrict__ subs, int P, const int64_t* __restrict__ rowptr,
                             const int32_t* __restrict__ colind, const double* __restrict__ vals,
                             const double* __restrict__ S, const double* __restrict__ ahat_diag,
                             const double* __restrict__ X, const double* __restrict__ theta, int ncheck,
-                            double sigma, double* __restrict__ resid) {
+                            double sigma, int d, double* __restrict__ gap, double* __restrict__ resid) {
     // thread t: column t % P (P is a power of two, at most 32) of every
     // (256 / P)-th row, so that a row's columns are read together; one
     // reciprocal of S per row (one per entry took most of the kernel's time)
@@ -616,10 +632,25 @@ __global__ void k_eig_resid(const SubInfo* __restrict__ subs, int P, const int64
     if (threadIdx.x == 0)
         for (int q = 0; q < kmax; ++q) worst = fmax(worst, sqrt(red[q]));
     if (threadIdx.x == 0) {
-        resid[blockIdx.x] = worst;
         const double* th = theta + (int64_t)blockIdx.x * P;
         const double lo = Sb.p > 0 ? th[0] + sigma : 1.0, hi = Sb.p > 0 ? th[Sb.p - 1] + sigma : 1.0;
-        resid[gridDim.x + blockIdx.x] = lo > 0.0 ? hi / lo : INFINITY;
+        double g = gap[blockIdx.x];
+        if (d >= 2 && Sb.p < Sb.n && lo > 0.0 && worst > 1e-13) {
+            const double x = 2.0 * g * hi / (th[kmax - 1] + sigma) - 1.0;
+            const double gr = d == 2 ? 2.0 * x * x - 1.0 : (4.0 * x * x - 3.0) * x;
+            const double v = worst / resid[blockIdx.x] * gr;
+            if (v > 1.0) {
+                const double told = 2.0 * g / (cosh(acosh(v) / d) + 1.0);
+                if (g > 1.0 && told < 1.5) gap[gridDim.x + blockIdx.x] = 0.0;
+                g = told;
+            } else if (gr < (d == 2 ? 4.0 : 8.0) && gap[gridDim.x + blockIdx.x] != 0.0) {
+                g *= 2.0;
+            }
+            g = g >= 1.0 ? fmin(g, kMaxGap) : 1.0;
+            gap[blockIdx.x] = g;
+        }
+        resid[blockIdx.x] = worst;
+        resid[gridDim.x + blockIdx.x] = lo > 0.0 ? g * hi / lo : INFINITY;
     }
 }
 
@@ -791,15 +822,16 @@ void launch_eig_update(cudaStream_t s, int64_t nrows_pad, int P, const int32_t* 
 void launch_eig_resid(cudaStream_t s, int nsub, const SubInfo* subs, int P, const int64_t* rowptr,
                       const int32_t* colind, const double* vals, const double* S,
                       const double* ahat_diag, const double* X, const double* theta, int ncheck,
-                      double sigma, double* resid) {
-    k_eig_resid<<<nsub, 256, 0, s>>>(subs, P, rowptr, colind, vals, S, ahat_diag, X, theta, ncheck, sigma, resid);
+                      double sigma, int d, double* gap, double* resid) {
+    k_eig_resid<<<nsub, 256, 0, s>>>(subs, P, rowptr, colind, vals, S, ahat_diag, X, theta, ncheck, sigma, d, gap,
+                                     resid);
 }
 void launch_eig_cheb(cudaStream_t s, int64_t nrows_pad, int P, const int32_t* sub_of_row, const SubInfo* subs,
-                     const double* theta, double sigma, double k, const double* w, double a, const double* u,
-                     double b, const double* v, double* out) {
+                     const double* theta, const double* gap, double sigma, double k, const double* w, double a,
+                     const double* u, double b, const double* v, double* out) {
     const int64_t tot = nrows_pad * P;
-    k_eig_cheb<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(nrows_pad, P, sub_of_row, subs, theta, sigma, k, w, a, u,
-                                                             b, v, out);
+    k_eig_cheb<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(nrows_pad, P, sub_of_row, subs, theta, gap, sigma, k, w, a,
+                                                             u, b, v, out);
 }
 void launch_eig_finalize(cudaStream_t s, int nsub, const SubInfo* subs, int P, const double* X,
                          const double* S, double* psi64) {

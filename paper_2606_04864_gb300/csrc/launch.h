@@ -256,11 +256,11 @@ void launch_eig_update(cudaStream_t s, int64_t nrows_pad, int P, const int32_t* 
 void launch_eig_resid(cudaStream_t s, int nsub, const SubInfo* subs, int P, const int64_t* rowptr,
                       const int32_t* colind, const double* vals, const double* S,
                       const double* ahat_diag, const double* X, const double* theta, int ncheck,
-                      double sigma, double* resid);
-// out = k (theta_p + sigma) w - a u - b v per subdomain (u may be NULL)
+                      double sigma, int d, double* gap, double* resid);
+// out = k gap (theta_p + sigma) w - a u - b v per subdomain (u may be NULL)
 void launch_eig_cheb(cudaStream_t s, int64_t nrows_pad, int P, const int32_t* sub_of_row, const SubInfo* subs,
-                     const double* theta, double sigma, double k, const double* w, double a, const double* u,
-                     double b, const double* v, double* out);
+                     const double* theta, const double* gap, double sigma, double k, const double* w, double a,
+                     const double* u, double b, const double* v, double* out);
 void launch_eig_finalize(cudaStream_t s, int nsub, const SubInfo* subs, int P, const double* X,
                          const double* S, double* psi64);
 void launch_psi_round(cudaStream_t s, int64_t n, const double* psi64, int prec, double* psi_used,
