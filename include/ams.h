@@ -85,7 +85,7 @@ typedef struct {
                                     side and keep the fastest */
     int32_t coarse;              /* 1: two-level (default); 0: local solves only */
     double eig_shift;            /* shift sigma of the local eigensolver; 0 = default 1e-2 */
-    int32_t eig_maxit;           /* local eigensolver iteration cap; 0 = default 300 */
+    int32_t eig_maxit;           /* cap on the local eigensolver's solves; 0 = default 300 */
     double eig_tol;              /* local eigenpair residual target; 0 = default 1e-13 */
     int64_t spin_budget_cycles;  /* budget of every bounded device-side wait
                                     (the local solves' mbarrier waits for
@@ -320,7 +320,9 @@ typedef struct {
     double setup_seconds;        /* wall time of ams_setup* */
     double eig_seconds;          /* of which: local eigensolves */
     double coarse_seconds;       /* of which: Galerkin product + coarse factor */
-    int32_t eig_iterations;      /* subspace iterations the eigensolver used */
+    int32_t eig_iterations;      /* shift-invert solves of the whole block the
+                                    eigensolver used (each filter step takes two
+                                    or three) */
     double eig_max_residual;     /* largest ||\hat A psi - lambda S psi||_{S^-1} kept */
     int64_t local_factor_bytes;  /* bytes of the stored local factors */
     int64_t coarse_inverse_bytes;/* bytes of the stored coarse inverse blocks */

@@ -560,6 +560,18 @@ __global__ void k_eig_update(int64_t nrows_pad, int P, const int32_t* __restrict
     X[t] = v;
 }
 
+// The P columns of a block (fewer rows than that: all of them) into the first
+// ones of a block of Q; the others are k_eig_init's.
+__global__ void k_eig_widen(int64_t nrows_pad, const int32_t* __restrict__ sub_of_row,
+                            const SubInfo* __restrict__ subs, int P, const double* __restrict__ X, int Q,
+                            double* __restrict__ out) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nrows_pad * P) return;
+    const int64_t row = t / P;
+    const int a = (int)(t % P), s = sub_of_row[row];
+    if (s >= 0 && a < subs[s].n) out[row * Q + a] = X[t];
+}
+
 // One step of the Chebyshev recurrence of the filtered subspace iteration, per
 // row of a subdomain with largest Ritz value theta_p and gap g (k_eig_resid):
 //   out = k g (theta_p + sigma) w - a u - b v   (u may be NULL; out may be w, u or v)
@@ -818,6 +830,11 @@ void launch_eig_update(cudaStream_t s, int64_t nrows_pad, int P, const int32_t* 
                        const SubInfo* subs, const double* Y, const double* T, double* X) {
     const int64_t tot = nrows_pad * P;
     k_eig_update<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(nrows_pad, P, sub_of_row, subs, Y, T, X);
+}
+void launch_eig_widen(cudaStream_t s, int64_t nrows_pad, const int32_t* sub_of_row, const SubInfo* subs, int P,
+                      const double* X, int Q, double* out) {
+    const int64_t tot = nrows_pad * P;
+    k_eig_widen<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(nrows_pad, sub_of_row, subs, P, X, Q, out);
 }
 void launch_eig_resid(cudaStream_t s, int nsub, const SubInfo* subs, int P, const int64_t* rowptr,
                       const int32_t* colind, const double* vals, const double* S,

@@ -257,6 +257,9 @@ void launch_eig_resid(cudaStream_t s, int nsub, const SubInfo* subs, int P, cons
                       const int32_t* colind, const double* vals, const double* S,
                       const double* ahat_diag, const double* X, const double* theta, int ncheck,
                       double sigma, int d, double* gap, double* resid);
+// the columns of a block of P into the first ones of a block of Q (d_esubs: with the wider p)
+void launch_eig_widen(cudaStream_t s, int64_t nrows_pad, const int32_t* sub_of_row, const SubInfo* subs, int P,
+                      const double* X, int Q, double* out);
 // out = k gap (theta_p + sigma) w - a u - b v per subdomain (u may be NULL)
 void launch_eig_cheb(cudaStream_t s, int64_t nrows_pad, int P, const int32_t* sub_of_row, const SubInfo* subs,
                      const double* theta, const double* gap, double sigma, double k, const double* w, double a,

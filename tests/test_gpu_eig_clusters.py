@@ -49,3 +49,18 @@ def test_no_more_solves_than_plain_steps(per, contrast, m):
     assert info["eig_max_residual"] <= 1e-11
     assert info["eig_iterations"] <= 48
     assert err <= 1e-11
+
+
+# More islands than the block has columns: it is widened to 32 after 56 solves and converges; 25 islands are held by 32
+# columns, 64 by none.  A cap below that leaves the block as it is.
+@pytest.mark.parametrize("per,m", [(5, 2), (5, 6), (5, 8), (8, 6)])
+def test_clusters_wider_than_the_block(per, m):
+    w = _islands(per, 1e4, m)
+    info, err = _solve(w)
+    assert info["eig_iterations"] < 300
+    assert info["eig_max_residual"] <= 1e-11
+    assert err <= 1e-11
+    for cap in (56, 57):
+        s = AmsSolver(w.rowptr, w.colind, w.vals, w.part, w.nparts, w.m, precision="fp64", eig_maxit=cap)
+        assert s.info()["eig_iterations"] == cap
+        assert all(np.isfinite(p).all() for p in s.coarse_basis()[2])
