@@ -1894,6 +1894,9 @@ static ams_status autotune(ams_handle h, const double* f_dev, int nrhs, int ld) 
         float best = 1e30f;
         int arg = T.bps_sub;
         for (int bps : cand_bps) {
+            // FP64: three, which is the fastest in a solve or within 2 % of it; back-to-back launches, which find
+            // their operands in L2, favour four or six (480^2 x 1 54 us at three, 66 at four; x 4 92 and 120)
+            if (h->prec == AMS_PREC_FP64 && bps != 3) continue;
             T.bps_sub = bps;
             AMS_TRY(ctx(&L));
             float ms = 0.f;

@@ -246,8 +246,17 @@ struct RowWords {
 // the loads free of branches (the mode as a run-time argument: 128^3 x 32 785
 // us, 96x80x72 x 3 78; this 735 and 72) and 64 registers, four blocks per SM
 // (two elements and six blocks 803 and 79, one and eight 834 and 79).
+// Blocks per SM that the registers are cut for: three where four spill and that
+// costs more than the fourth block gives.  us a launch at four / three: 96^3 with
+// 10 modes x 1 86 / 71, x 4 195 / 170, but x 16 212 / 229; 480^2 with 12 modes in
+// FP64 x 8 104 / 91; in chunks with an FP32 basis, 48^3 in 4^3 blocks x 32 138 / 122.
+template <typename TF, typename TP, int LD, int MM, bool CH>
+constexpr int prolong_blocks() {
+    if (CH) return MM > 8 || sizeof(TP) == 4 ? 3 : 4;
+    return MM > 8 && (sizeof(TF) == 8 || LD <= 4) ? 3 : 4;
+}
 template <typename TF, typename TP, int LD, int MM, int MODE, bool CH>
-__global__ void __launch_bounds__(kRedThreads, 4)
+__global__ void __launch_bounds__(kRedThreads, prolong_blocks<TF, TP, LD, MM, CH>())
 k_prolong_update(const SubInfo* __restrict__ subs, const TP* __restrict__ psi, const TF* __restrict__ ec,
                  const TF* __restrict__ yc, const TF* __restrict__ qmat, const CoarseRef* __restrict__ cref, const int32_t* __restrict__ gat,
                  const TF* __restrict__ zf, double* __restrict__ r, const double* __restrict__ q,
