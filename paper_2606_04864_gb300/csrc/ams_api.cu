@@ -1417,6 +1417,11 @@ static int local_extra_launches(ams_handle h, int ld) {
     return (int)h->cls_c.size() - 1;
 }
 
+static LocalSolveArgs local_solve_args(ams_handle h, int ld, const ResidIn& in, bool with_state) {
+    return LocalSolveArgs{h->stream, h->N, h->d_subs, in, nullptr, ld, h->cmax, std::max(1, h->mmax),
+                          with_state ? h->d_st : nullptr, h->use_pdl, h->tune[ld].depth, h->ncols, h->num_sms};
+}
+
 static ams_status launch_local(ams_handle h, int ld, const ResidIn& in, bool with_state,
                                bool restrict_rc = true) {
     const bool coarse = h->Nc > 0 && restrict_rc;
@@ -1424,11 +1429,8 @@ static ams_status launch_local(ams_handle h, int ld, const ResidIn& in, bool wit
         LocalTmaArgs a = local_tma_args(h, ld, in, with_state);
         AMS_CUDA_TRY(launch_local_tma(a, h->prec, h->d_psi, h->d_psif, h->d_zf, coarse ? h->d_rc : nullptr));
     } else {
-        LocalSolveArgs la{h->stream, h->N, h->d_subs, in, nullptr, ld, h->cmax, std::max(1, h->mmax),
-                          with_state ? h->d_st : nullptr, h->use_pdl, h->tune[ld].depth, h->ncols,
-                          h->num_sms};
-        AMS_CUDA_TRY(launch_local_solve(la, (const double*)h->d_fac, (const double*)h->d_psi, (double*)h->d_zf,
-                                        coarse ? (double*)h->d_rc : nullptr));
+        AMS_CUDA_TRY(launch_local_solve(local_solve_args(h, ld, in, with_state), (const double*)h->d_fac,
+                                        (const double*)h->d_psi, (double*)h->d_zf, coarse ? (double*)h->d_rc : nullptr));
     }
     return AMS_OK;
 }
@@ -1846,17 +1848,19 @@ static ams_status autotune(ams_handle h, const double* f_dev, int nrhs, int ld) 
     };
     {   // local-solve ring depth (staging within 200 KB) and right-hand sides per column group together:
         // the right depth depends on the group's size.  The right-looking kernels (all but the one-RHS
-        // one) gain nothing from more than a few rows in flight and lose occupancy to them.
+        // one and the FP64 lane-per-row one) gain nothing from more than a few rows in flight and lose
+        // occupancy to them.
         const ResidIn in{h->d_r, h->d_q, h->d_sc};
         const bool one_rhs = h->use_tma && ld == 1;
         const int nr_hi = !h->use_tma ? 0 : ld >= 16 ? 16 : ld == 4 ? 4 : 0, nr_lo = nr_hi / 2;   // 0: no choice
-        const int dmin = h->use_tma ? 2 : 1, dmax = one_rhs ? 6 : h->use_tma ? 4 : 3;
+        const int dmin = h->use_tma ? 2 : 1;
+        const int dmax = one_rhs ? 6 : h->use_tma ? 4 : local_solve_max_depth(local_solve_args(h, ld, in, true));
         float best = 1e30f;
         int arg = 0, argn = 0;
         for (int nr = nr_hi; nr >= nr_lo; nr = nr > nr_lo ? nr_lo : -1) {
             for (int d = dmin; d <= dmax; ++d) {
                 const size_t smem = h->use_tma ? local_tma_launch_smem(local_tma_args(h, ld, in, true), d)
-                                               : local_solve_smem(h->cmax, ld, h->tf_bytes(), d);
+                                               : local_solve_launch_smem(local_solve_args(h, ld, in, true), d);
                 if (smem > 200 * 1024) continue;
                 T.depth = d;
                 T.nr = nr;

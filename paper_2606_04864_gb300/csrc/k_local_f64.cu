@@ -630,17 +630,42 @@ static cudaError_t local_f64_rows(const LocalSolveArgs& a, const double* fac, co
                          a.in.sc, a.rowscale, zf, psi, rc, a.ld, a.cmax, depth, a.st);
 }
 
+// A lane per row where the FP64 pipe is full: one tile a block row and enough
+// subdomains.  Lane per row / row pairs, us a launch at 1, 2, 3, 4 columns, the
+// subdomains an SM in brackets, the better ring depth of each:
+//   up to 8 modes
+//     256 of 16^2 (1.7)    62 / 62   112 / 79   194 / 102  174 / 95
+//     441 of 16^2 (2.9)    65 / 81   106 / 94   178 / 120  199 / 139
+//     484 of 32^2 (3.2)   262 / 376  444 / 462  778 / 666  778 / 699
+//     529 of 16^2 (3.5)    65 / 96   112 / 122  198 / 172  199 / 176
+//     625 of 16^2 (4.1)    69 / 151  118 / 145  194 / 250  194 / 201
+//     1024 of 32^2 (6.7)  286 / 711  512 / 860  967 / 1123 967 / 1303
+//   more
+//     121 of 32^2 (0.8)   274 / 233  429 / 255  427 / 277  427 / 343
+//     196 of 32^2 (1.3)   274 / 286  453 / 332  452 / 449  452 / 444
+//     361 of 12^2 (2.4)    47 / 61    77 / 75    87 / 146   82 / 92
+//     625 of 16^2 (4.1)    75 / 180  112 / 195  223 / 296  238 / 282
+// With two tiles a block row the pairs are the faster at any number (1728 of 8^3,
+// 11 an SM: 395 / 379, 1230 / 884, 2156 / 1305, 2156 / 1403).
+static bool f64_by_rows(const LocalSolveArgs& a) {
+    if (a.cmax != 1 || a.ld > 4) return false;
+    const bool big = a.mmax > 8;
+    const int per_sm = a.ld == 1 ? (big ? 1 : 2) : a.ld == 2 ? 3 : big ? 2 : 4;
+    return a.nsub > per_sm * a.sms;
+}
+
+// Ring depths worth trying, and what one takes: the left-looking kernel gains
+// from up to six (480^2 in 16^2 blocks, 12 modes x 3: 290 us at three, 233 at five),
+// the other one from a few.
+int local_solve_max_depth(const LocalSolveArgs& a) { return f64_by_rows(a) ? 6 : 3; }
+size_t local_solve_launch_smem(const LocalSolveArgs& a, int depth) {
+    return f64_by_rows(a) ? local_solve_smem(a.cmax, a.ld, 8, depth) : local_f64_smem(a.cmax, a.ncols, depth);
+}
+
 template <int MM>
 static cudaError_t local_f64_mm(const LocalSolveArgs& a, const double* fac, const double* psi, double* zf, double* rc) {
-    // A lane per row where the FP64 pipe is full: one tile a block row and enough
-    // subdomains.  Lane per row / row pairs, us a launch at 1, 2, 3, 4 columns:
-    //   1024 subdomains of 32^2 (6.7 an SM)  293 / 730  512 / 860  967 / 1122  967 / 1304
-    //   361 of 16^2 (2.4)                     40 / 49   104 / 92   179 / 122   179 / 128
-    //   256 of 32^2 (1.7)                    247 / 238  430 / 288  758 / 387   758 / 402
-    //   1728 of 8^3 (11, two tiles)          395 / 379 1230 / 884 2156 / 1305 2156 / 1403
-    //   512 of 8^3 (3.4, two tiles)          199 / 131  597 / 298 1050 / 430  1050 / 461
     constexpr int R4 = MM > 8 ? 2 : 4;   // columns a warp (registers)
-    if (a.cmax == 1 && a.ld <= 4 && a.nsub > (a.ld == 1 ? 2 : 4) * a.sms) {
+    if (f64_by_rows(a)) {
         if (a.ld == 1) return local_f64_rows<1, MM>(a, fac, psi, zf, rc);
         if (a.ld == 2) return local_f64_rows<2, MM>(a, fac, psi, zf, rc);
         return local_f64_rows<R4, MM>(a, fac, psi, zf, rc);

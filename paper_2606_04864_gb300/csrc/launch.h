@@ -149,7 +149,9 @@ void launch_dir_update(const LaunchCtx& L, int prec, const void* z, const double
 void launch_x_flush(const LaunchCtx& L, const double* p, const double* p2, double* x);
 void launch_init_norms(const LaunchCtx& L, const double* r, int nrhs);
 size_t local_solve_smem(int cmax, int ld, size_t tf_bytes, int depth);
-// FP64 local solves (k_local_f64.cu)
+// FP64 local solves (k_local_f64.cu); the deepest ring that the kernel chosen for `a` may gain from, and its shared memory
+int local_solve_max_depth(const LocalSolveArgs& a);
+size_t local_solve_launch_smem(const LocalSolveArgs& a, int depth);
 cudaError_t launch_local_solve(const LocalSolveArgs& a, const double* fac, const double* psi, double* zf, double* rc);
 void launch_coarse_gemm(const CoarseLaunch& c, int prec, int ld, const void* in, void* out);
 // The launch uses the one-vector kernel (one launch whatever the band widths).
