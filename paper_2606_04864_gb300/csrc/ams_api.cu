@@ -1895,12 +1895,17 @@ static ams_status autotune(ams_handle h, const double* f_dev, int nrhs, int ld) 
         T.l2keep = cand[arg][1];
     }
     {   // subdomain layout: prolongation (updates x and r of this throw-away state)
+        auto filled = [&](int bps) {   // subdomains of a block, on average of the most
+            const double avg = (double)h->N / (bps * h->num_sms);
+            return avg / std::ceil(avg);
+        };
         float best = 1e30f;
         int arg = T.bps_sub;
         for (int bps : cand_bps) {
             // FP64: three, which is the fastest in a solve or within 2 % of it; back-to-back launches, which find
-            // their operands in L2, favour four or six (480^2 x 1 54 us at three, 66 at four; x 4 92 and 120)
-            if (h->prec == AMS_PREC_FP64 && bps != 3) continue;
+            // their operands in L2, favour four or six (480^2 x 1 54 us at three, 66 at four; x 4 92 and 120).
+            // Others only where whole subdomains fill their blocks a quarter better (576 of them x 3 153 and 115)
+            if (h->prec == AMS_PREC_FP64 && filled(bps) <= 1.25 * filled(3) && bps != 3) continue;
             T.bps_sub = bps;
             AMS_TRY(ctx(&L));
             float ms = 0.f;
