@@ -165,7 +165,7 @@ struct ams_handle_s {
     int32_t* d_cnt = nullptr;
     // solve work space (sized for ld_alloc)
     int ld_alloc = 0, ld_last = 0;
-    int ncols = 1;              // right-hand sides of the current call
+    int ncols = 1;              // right-hand sides of the current (or last) call
     double *d_x = nullptr, *d_r = nullptr, *d_p = nullptr, *d_q = nullptr, *d_z = nullptr;
     double* d_p2 = nullptr;             // second direction buffer (iterations alternate p and p2)
     void *d_zf = nullptr, *d_rc = nullptr, *d_yc = nullptr, *d_ec = nullptr;
@@ -2135,11 +2135,10 @@ ams_status ams_destroy(ams_handle h) {
     return AMS_OK;
 }
 
-// Algorithmic bytes of one launch of kernel `which` (each operand read once,
-// each output written once) at `ld` right-hand sides.
-// Algorithmic bytes of one launch: every operand read once, every output
-// written once (FP64 vectors, the stored factor and basis at their storage
-// precision).
+// Algorithmic bytes of one launch of kernel `which` at stride `ld`: every operand
+// read once, every output written once (FP64 vectors, the stored factor and
+// basis at their storage precision).  The FP64 local solves run for the last
+// call's right-hand sides, everything else for the stride.
 static double kernel_bytes(ams_handle h, int which, int ld) {
     const double n = (double)h->n_total, nl = n * ld;
     const double tf = (double)h->tf_bytes(), tp = (double)h->tp_bytes();
@@ -2152,7 +2151,8 @@ static double kernel_bytes(ams_handle h, int which, int ld) {
             // factor once (tiles + pivots, or the packed factor), r and q in,
             // z_f out, basis rows, r_c out
             const double fb = h->use_tma ? (double)h->tile_elems * 4.0 + 4.0 * n : (double)h->fac_elems * tf;
-            return fb + 16.0 * nl + tf * nl + (double)h->psi_elems * tp + (double)h->Nc * ld * tf;
+            const double cols = h->use_tma ? ld : h->ncols;
+            return fb + (16.0 + tf) * n * cols + (double)h->psi_elems * tp + (double)h->Nc * cols * tf;
         }
         case AMS_KERNEL_COARSE:     // forward blocks, r_c in, y out (+ the backward pass when separate)
             return (double)h->R_elems * tf + 2.0 * (double)h->Nc * ld * tf +
@@ -2500,6 +2500,7 @@ ams_status ams_spmv(ams_handle h, const double* x, int32_t nrhs, double* y) {
         return AMS_ERR_INVALID_ARG;
     }
     const int ld = pow2ceil(nrhs);
+    h->ncols = nrhs;
     AMS_TRY(ensure_work(h, ld));
     RedCache *rc = nullptr, *rcs = nullptr;
     AMS_TRY(get_red(h, ld, &rc, &rcs));
@@ -2528,7 +2529,6 @@ ams_status ams_time_kernel(ams_handle h, int32_t which, int32_t reps, double* av
     }
     AMS_TRY(enter(h));
     const int ld = h->ld_last;
-    h->ncols = ld;
     RedCache *rc = nullptr, *rcs = nullptr;
     AMS_TRY(get_red(h, ld, &rc, &rcs));
     LaunchCtx L = make_ctx(h, *rc, *rcs);

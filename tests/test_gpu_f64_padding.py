@@ -110,3 +110,15 @@ def test_one_handle_with_one_count_after_another(cycle):
             assert abs(int(its[i]) - ref[i].iters) <= 2
             tol = 1e-10 if int(its[i]) == ref[i].iters else 1e-6
             assert np.linalg.norm(u[i] - ref[i].u) <= tol * np.linalg.norm(ref[i].u)
+
+
+def test_reported_bytes_are_those_of_the_columns_there_are():
+    w = make_small_3d(side=15, bs=8, m=4, std=1.5, seed=97)
+    s = AmsSolver(w.rowptr, w.colind, w.vals, w.part, w.nparts, w.m, precision="fp64")
+    f = np.random.default_rng(98).standard_normal((8, w.n))
+    per_column = 8 * (3 * w.n + s.info()["ncoarse"])   # r and q in, z_f and r_c out
+    local = {}
+    for nrhs in (8, 5, 7):
+        local[nrhs] = s.profile_solve(f[:nrhs])[1]["bytes"]
+        assert s.time_kernel(1, 1)[1] == local[nrhs]
+    assert local[8] - local[5] == 3 * per_column and local[8] - local[7] == per_column
