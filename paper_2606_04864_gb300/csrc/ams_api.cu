@@ -1895,17 +1895,28 @@ static ams_status autotune(ams_handle h, const double* f_dev, int nrhs, int ld) 
         T.l2keep = cand[arg][1];
     }
     {   // subdomain layout: prolongation (updates x and r of this throw-away state)
-        auto filled = [&](int bps) {   // subdomains of a block, on average of the most
-            const double avg = (double)h->N / (bps * h->num_sms);
-            return avg / std::ceil(avg);
-        };
+        // Steps of length zero from here on, with z = M^{-1} r: r stays and r.z stays positive.  Repeated real steps
+        // on one z soon make it negative, which ends a PCG solve as a breakdown; every later launch then returned at
+        // once, and the FP64 grids were chosen from 6 us noise (480^2 x 4: four blocks an SM, 117 us in the solve
+        // where three take 90).
+        std::vector<CgScalars> sc((size_t)h->nsys * ld);
+        AMS_CUDA_TRY(cudaMemcpyAsync(sc.data(), h->d_sc, sizeof(CgScalars) * sc.size(), cudaMemcpyDeviceToHost,
+                                     h->stream));
+        SolveState st{};
+        AMS_CUDA_TRY(cudaMemcpyAsync(&st, h->d_st, sizeof(st), cudaMemcpyDeviceToHost, h->stream));
+        AMS_CUDA_TRY(cudaStreamSynchronize(h->stream));
+        for (auto& c : sc) c.alpha = 0.0;
+        st.done = 0;
+        st.status = 0;
+        AMS_CUDA_TRY(cudaMemcpyAsync(h->d_sc, sc.data(), sizeof(CgScalars) * sc.size(), cudaMemcpyHostToDevice,
+                                     h->stream));
+        AMS_CUDA_TRY(cudaMemcpyAsync(h->d_st, &st, sizeof(st), cudaMemcpyHostToDevice, h->stream));
+        AMS_TRY(local_pre());
+        if (h->Nc > 0) launch_coarse(h, ld, true);
+        AMS_CUDA_TRY(cudaStreamSynchronize(h->stream));
         float best = 1e30f;
         int arg = T.bps_sub;
         for (int bps : cand_bps) {
-            // FP64: three, which is the fastest in a solve or within 2 % of it; back-to-back launches, which find
-            // their operands in L2, favour four or six (480^2 x 1 54 us at three, 66 at four; x 4 92 and 120).
-            // Others only where whole subdomains fill their blocks a quarter better (576 of them x 3 153 and 115)
-            if (h->prec == AMS_PREC_FP64 && filled(bps) <= 1.25 * filled(3) && bps != 3) continue;
             T.bps_sub = bps;
             AMS_TRY(ctx(&L));
             float ms = 0.f;
