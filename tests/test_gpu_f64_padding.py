@@ -9,7 +9,7 @@ import pytest
 from oracle import OracleAMS, csr_to_scipy, pcg
 from workloads import make_small_3d
 
-from .native import run_native
+from .native import build_native, run_native
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -83,11 +83,16 @@ int main(int, char** argv) {
 """
 
 
+@pytest.fixture(scope="module")
+def program(tmp_path_factory):
+    return build_native(tmp_path_factory.mktemp("native"), SOURCE)
+
+
 # row pairs with every number of lanes a task, and (700 subdomains, up to four columns) a lane per row
 @pytest.mark.parametrize("ncols,ld,nsub", [(1, 1, 2), (2, 2, 2), (3, 4, 2), (5, 8, 2), (7, 8, 2), (9, 16, 2), (17, 32, 2),
                                            (31, 32, 2), (32, 32, 2), (3, 4, 700)])
-def test_columns_without_a_right_hand_side_are_zero(tmp_path, ncols, ld, nsub):
-    assert run_native(tmp_path, SOURCE, ncols, ld, nsub) == ["0"]
+def test_columns_without_a_right_hand_side_are_zero(program, ncols, ld, nsub):
+    assert run_native(program, ncols, ld, nsub) == ["0"]
 
 
 @pytest.mark.parametrize("cycle", [False, True])

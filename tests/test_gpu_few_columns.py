@@ -15,7 +15,7 @@ pytestmark = pytest.mark.gpu
 if not torch.cuda.is_available():  # pragma: no cover
     pytest.skip("no CUDA device", allow_module_level=True)
 
-from paper_2606_04864_gb300 import AmsSolver  # noqa: E402
+from paper_2606_04864_gb300 import AmsError, AmsSolver  # noqa: E402
 
 
 def _grid(nx, ny, shift):
@@ -92,3 +92,17 @@ def test_launch_count_with_two_band_widths():
         s.apply_preconditioner(r[:nrhs])
         counts.append(s.info()["kernel_launches"] - before)
     assert counts[0] == counts[1] == 5   # two permutes, two band widths, the prolongation
+
+
+@pytest.mark.parametrize("nrhs", [2, 4])
+def test_exhausted_wait_reports_timeout_and_the_next_handle_solves(nrhs):
+    """Every block first waits, for a short budget, on a barrier that nothing completes."""
+    w = make_small_2d(side=48, bs=8, m=3, std=1.5, seed=78)
+    f = np.random.default_rng(9).standard_normal((nrhs, w.n))
+    args = (w.rowptr, w.colind, w.vals, w.part, w.nparts, w.m)
+    s = AmsSolver(*args, precision="fp32", autotune=False, spin_budget_cycles=20000, timeout_probe=True)
+    with pytest.raises(AmsError) as e:
+        s.apply_preconditioner(f)
+    assert e.value.status == 5   # AMS_ERR_DEVICE_TIMEOUT
+    u, _, rel = AmsSolver(*args, precision="fp32", autotune=False).solve(f)
+    assert (rel <= 1e-8).all()

@@ -2,7 +2,7 @@
 the right-hand-side strides whose kernels are compiled with them.  No launch:
 the calls have no subdomains."""
 
-from .native import run_native
+from .native import build_native, run_native
 
 SOURCE = r"""
 #include <cstdio>
@@ -28,6 +28,6 @@ int main() {
 
 
 def test_strides_without_the_code_refuse_the_arguments(tmp_path):
-    got = {tuple(map(int, line.split())) for line in run_native(tmp_path, SOURCE)}
+    got = {tuple(map(int, line.split())) for line in run_native(build_native(tmp_path, SOURCE))}
     assert got == {(ld, q, x, int((q and ld > 4) or (not x and ld < 8)))
                    for ld in (1, 2, 4, 8, 16, 32) for q in (0, 1) for x in (0, 1)}

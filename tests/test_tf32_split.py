@@ -3,7 +3,7 @@ and together they are the operand to one unit of FP32."""
 
 import numpy as np
 
-from .native import run_native
+from .native import build_native, run_native
 
 SOURCE = r"""
 #include <cmath>
@@ -38,7 +38,7 @@ int main() {
 
 
 def test_parts_are_tf32_and_sum_to_the_operand(tmp_path):
-    assert run_native(tmp_path, SOURCE) == ["0 0 0 1"]
+    assert run_native(build_native(tmp_path, SOURCE)) == ["0 0 0 1"]
 
 
 def test_products_of_split_operands():
