@@ -52,9 +52,9 @@
 // per column group); column groups share only the tiles.
 //
 // Measured (us a launch, row-major kernel with one warp per 8 columns before):
-// 128^3 x 32 1224 -> 711-750, 96^3 x 16 314 -> 183, 8 uneven systems x 8
+// 128^3 x 32 1224 -> 613-667, 96^3 x 16 314 -> 178, 8 uneven systems x 8
 // 406 -> 172, 77^3 x 8 (cycle, with its scaling) 222 -> 105, 64^3 x 8 91 -> 57.  One warp per column group with both row
-// halves: 32: 742, 16: 191, 8 uneven systems 192, 64^3 x 8 68.
+// halves: 742, 191, 192 and (64^3 x 8) 68.
 #include <algorithm>
 #include <cstdint>
 
